@@ -259,6 +259,7 @@ __device__ __forceinline__ int fine_scan(const WF& wf, int v_lo, int v_hi, float
         if (running + before <= target) {     // warp-uniform; the warps after the one that holds the target stay out
             const float lo = running + (before + (inc - ls));
             const unsigned crossing = __ballot_sync(0xffffffffu, ls > 0.f && lo + ls > target);
+            unsigned some = 0;
             if (crossing) {
                 // lane (k, j) = (lane / EPV, lane % EPV) takes element j of vector k of the crossing run
                 const int src = __ffs(crossing) - 1;
@@ -266,11 +267,12 @@ __device__ __forceinline__ int fine_scan(const WF& wf, int v_lo, int v_hi, float
                 const int vi = __shfl_sync(0xffffffffu, first, src) + lane / EPV;
                 const float e = lane / EPV < run && vi < v_hi ? wf.element(vi, lane % EPV) : 0.f;
                 const float cum = start + warp_scan_incl(e, lane);
-                const unsigned some = __ballot_sync(0xffffffffu, e > 0.f);
+                some = __ballot_sync(0xffffffffu, e > 0.f);
                 const unsigned over = __ballot_sync(0xffffffffu, e > 0.f && cum > target);
                 if (lane == (over ? __ffs(over) - 1 : 31 - __clz(some)))
                     atomicMin(&sh.key, static_cast<unsigned>(vi * EPV + lane % EPV));
-            } else {
+            }
+            if (!some) {      // also where a run has a sum at rounding level but no element of its own
                 const int lv = __reduce_max_sync(0xffffffffu, lastv);
                 if (lane == 0 && lv >= 0) atomicMax(&sh.lastpos, lv);
             }

@@ -47,7 +47,8 @@ struct TreeArgs {
 
 // Weights of the distribution after `nrej` rejections at a node, unnormalised: p for nrej == 0, else
 // max(0, p_nrej - q) with p_1 = p and p_{i+1} = max(0, p_i - q) * rS[i].  Few members: registers are what the passes
-// over the rows run short of.
+// over the rows run short of.  Every operation is rounded by itself, so that of(), weights() and element() give the same
+// number where a residual is at rounding level.
 template <int DT>
 struct TreeWeights {
     RowGeom gt;
@@ -60,8 +61,8 @@ struct TreeWeights {
         if (nrej == 0) return p;
         float r = p;
 #pragma unroll 1
-        for (int i = 1; i < nrej; ++i) r = fmaxf(r - q, 0.f) * rS[i];
-        return fmaxf(r - q, 0.f);
+        for (int i = 1; i < nrej; ++i) r = __fmul_rn(fmaxf(__fsub_rn(r, q), 0.f), rS[i]);
+        return fmaxf(__fsub_rn(r, q), 0.f);
     }
     // The draft row starts at the same 16-byte phase as the target row.
     __device__ __forceinline__ bool same_phase() const {
@@ -80,7 +81,7 @@ struct TreeWeights {
         unpack_masked<DT>(raw.t, vi, gt, w);
 #pragma unroll
         for (int j = 0; j < EPV; ++j)      // NaN / -inf: no mass
-            w[j] = ex2_approx(fmaxf(__fmaf_rn(w[j], c, -Mp), kArgFloor)) * rZp;
+            w[j] = __fmul_rn(ex2_approx(fmaxf(__fmaf_rn(w[j], c, -Mp), kArgFloor)), rZp);
         if (nrej == 0) return;
         float q[EPV];
         if (same_phase()) {
@@ -93,23 +94,23 @@ struct TreeWeights {
             }
         }
 #pragma unroll
-        for (int j = 0; j < EPV; ++j) q[j] = ex2_approx(fmaxf(__fmaf_rn(q[j], c, -Mq), kArgFloor)) * rZq;
+        for (int j = 0; j < EPV; ++j) q[j] = __fmul_rn(ex2_approx(fmaxf(__fmaf_rn(q[j], c, -Mq), kArgFloor)), rZq);
 #pragma unroll 1
         for (int i = 1; i < nrej; ++i) {
             const float s = rS[i];
 #pragma unroll
-            for (int j = 0; j < EPV; ++j) w[j] = fmaxf(w[j] - q[j], 0.f) * s;
+            for (int j = 0; j < EPV; ++j) w[j] = __fmul_rn(fmaxf(__fsub_rn(w[j], q[j]), 0.f), s);
         }
 #pragma unroll
-        for (int j = 0; j < EPV; ++j) w[j] = fmaxf(w[j] - q[j], 0.f);
+        for (int j = 0; j < EPV; ++j) w[j] = fmaxf(__fsub_rn(w[j], q[j]), 0.f);
     }
     __device__ __forceinline__ float element(int vi, int j) const {
         const int i = vi * ElemTraits<DT>::kEPV + j - gt.pre;
         if (i < 0 || i >= gt.V) return 0.f;
         const char* trow = reinterpret_cast<const char*>(gt.base) + gt.pre * ElemTraits<DT>::kBytes;
-        const float p = ex2_approx(fmaxf(__fmaf_rn(ElemTraits<DT>::load_one(trow, i), c, -Mp), kArgFloor)) * rZp;
+        const float p = __fmul_rn(ex2_approx(fmaxf(__fmaf_rn(ElemTraits<DT>::load_one(trow, i), c, -Mp), kArgFloor)), rZp);
         float q = 0.f;
-        if (nrej > 0) q = ex2_approx(fmaxf(__fmaf_rn(ElemTraits<DT>::load_one(qrow, i), c, -Mq), kArgFloor)) * rZq;
+        if (nrej > 0) q = __fmul_rn(ex2_approx(fmaxf(__fmaf_rn(ElemTraits<DT>::load_one(qrow, i), c, -Mq), kArgFloor)), rZq);
         return of(p, q);
     }
 };

@@ -29,7 +29,9 @@ struct FinishArgs {
     int after_stats;              // verify_finish_kernel: row_stats_kernel is its predecessor (see svip_device.cuh)
 };
 
-// Weights max(0, p - q) of Algorithm 4 (or p alone for the bonus token) for one vector.
+// Weights max(0, p - q) of Algorithm 4 (or p alone for the bonus token) for one vector.  Products and difference are rounded
+// one by one, as in residual_segment_sum: a residual at rounding level is then the same number in the sum of the segment, in
+// the sum of a run and as an element.
 template <int DT>
 struct ResidualWeights {
     RowGeom gt, gq;
@@ -65,7 +67,7 @@ struct ResidualWeights {
         unpack_masked<DT>(raw.t, vi, gt, x);
 #pragma unroll
         for (int j = 0; j < EPV; ++j)
-            w[j] = x[j] >= thr_p ? ex2_approx(fmaxf(__fmaf_rn(x[j], c, -Mp), kArgFloor)) * rZp : 0.f;
+            w[j] = x[j] >= thr_p ? __fmul_rn(ex2_approx(fmaxf(__fmaf_rn(x[j], c, -Mp), kArgFloor)), rZp) : 0.f;
         if (bonus) return;
         float d[EPV];
         if (gq.pre == gt.pre) {
@@ -80,19 +82,19 @@ struct ResidualWeights {
         }
 #pragma unroll
         for (int j = 0; j < EPV; ++j) {
-            float q = d[j] >= thr_q ? ex2_approx(fmaxf(__fmaf_rn(d[j], c, -Mq), kArgFloor)) * rZq : 0.f;
-            w[j] = fmaxf(w[j] - q, 0.f);
+            float q = d[j] >= thr_q ? __fmul_rn(ex2_approx(fmaxf(__fmaf_rn(d[j], c, -Mq), kArgFloor)), rZq) : 0.f;
+            w[j] = fmaxf(__fsub_rn(w[j], q), 0.f);
         }
     }
     __device__ __forceinline__ float element(int vi, int j) const {
         const int i = vi * ElemTraits<DT>::kEPV + j - gt.pre;
         if (i < 0 || i >= gt.V) return 0.f;
         const float x = ElemTraits<DT>::load_one(trow, i);
-        const float p = x >= thr_p ? ex2_approx(fmaxf(__fmaf_rn(x, c, -Mp), kArgFloor)) * rZp : 0.f;
+        const float p = x >= thr_p ? __fmul_rn(ex2_approx(fmaxf(__fmaf_rn(x, c, -Mp), kArgFloor)), rZp) : 0.f;
         if (bonus) return p;
         const float d = ElemTraits<DT>::load_one(qrow, i);
-        const float q = d >= thr_q ? ex2_approx(fmaxf(__fmaf_rn(d, c, -Mq), kArgFloor)) * rZq : 0.f;
-        return fmaxf(p - q, 0.f);
+        const float q = d >= thr_q ? __fmul_rn(ex2_approx(fmaxf(__fmaf_rn(d, c, -Mq), kArgFloor)), rZq) : 0.f;
+        return fmaxf(__fsub_rn(p, q), 0.f);
     }
 };
 
