@@ -72,6 +72,9 @@ typedef enum {
 #define SVIP_STATUS_DEBUG_OOB 16u    /* bounds-checked build only: a kernel asked for logits outside the buffers
                                         of its call (the load was not performed) */
 
+#define SVIP_STATUS_LOOP_OVERLAP 32u /* two replays of drafting loops of one context ran at the same time: a loop was ended
+                                        early and the outputs of both are not valid */
+
 /* draft-side layout selector for svip_verify: rows packed sequence after sequence */
 #define SVIP_Q_PACKED (-1L)
 
@@ -536,6 +539,8 @@ int svip_graph_destroy(svip_graph* graph);
  * svip_policy_advance is recorded right after the svip_draft_step_at of the same
  * sequences (pos = draft_len, same active and stop), the draft kernel takes the
  * policy step and the decision as well: one kernel per drafted token.
+ * The loops of a context share its counters: replays that hold one must not
+ * overlap on the GPU (SVIP_STATUS_LOOP_OVERLAP).
  * One loop at a time (no nesting); svip_graph_end on a graph whose loop body
  * was not closed, or could not be recorded, returns SVIP_ERR_STATE and hands
  * out no graph.  Calls inside the body must come from the thread that opened

@@ -27,6 +27,7 @@ SVIP_STATUS_NONFINITE_ROW = 1
 SVIP_STATUS_BAD_DRAFT_LEN = 2
 SVIP_STATUS_WAIT_TIMEOUT = 4
 SVIP_STATUS_BAD_TREE = 8
+SVIP_STATUS_LOOP_OVERLAP = 32
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 # SVIP_LIBRARY in the environment points at another build of the same ABI (a debug build, say)

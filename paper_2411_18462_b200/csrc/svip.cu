@@ -61,8 +61,9 @@ struct svip_ctx {
     float2* q_stats;
     int32_t* p_argmax;
     unsigned* status;
-    int* loop_iter;            // device: iteration counter of the drafting loop being replayed
-    unsigned long long* loop_arrived;   // device: sequences counted by the draft kernel of that loop, zero between launches
+    unsigned long long* loop_arrived;   // device: sequences counted by the draft kernel of the drafting loop being replayed,
+                                        // zero between launches; behind it ...
+    int* loop_iter;                     // ... the iteration counter of that loop (both cleared when a replay enters it)
     cudaGraphNode_t loop_draft_node;    // the last draft step recorded in the loop body, if nothing came after it ...
     DraftArgs loop_draft_args;          // ... and its arguments
     int loop_draft_rows;
@@ -79,6 +80,7 @@ struct svip_ctx {
 };
 
 constexpr int kProfilePairs = 4096;
+constexpr size_t kLoopStateBytes = 16;    // loop_arrived and loop_iter
 
 struct svip_graph {
     cudaGraphExec_t exec;
@@ -362,17 +364,16 @@ int svip_create(svip_ctx** out, int device, int max_rows) {
             cudaMalloc(&c->p_argmax, n * sizeof(int32_t)) != cudaSuccess ||
             cudaMalloc(&c->status, sizeof(unsigned)) != cudaSuccess ||
             cudaMemset(c->status, 0, sizeof(unsigned)) != cudaSuccess ||
-            cudaMalloc(&c->loop_iter, sizeof(int)) != cudaSuccess ||
-            cudaMemset(c->loop_iter, 0, sizeof(int)) != cudaSuccess ||
-            cudaMalloc(&c->loop_arrived, sizeof(unsigned long long)) != cudaSuccess ||
-            cudaMemset(c->loop_arrived, 0, sizeof(unsigned long long)) != cudaSuccess) {
+            cudaMalloc(&c->loop_arrived, kLoopStateBytes) != cudaSuccess ||
+            cudaMemset(c->loop_arrived, 0, kLoopStateBytes) != cudaSuccess) {
             rc = SVIP_ERR_CUDA;
         }
+        c->loop_iter = reinterpret_cast<int*>(c->loop_arrived + 1);
     }
     if (rc != SVIP_OK) {
         cudaGetLastError();
         cudaFree(c->p_stats); cudaFree(c->q_stats); cudaFree(c->p_argmax); cudaFree(c->status);
-        cudaFree(c->loop_iter); cudaFree(c->loop_arrived);
+        cudaFree(c->loop_arrived);
         delete c;
     } else {
         *out = c;
@@ -387,7 +388,7 @@ int svip_destroy(svip_ctx* ctx) {
     cudaGetDevice(&prev);
     cudaSetDevice(ctx->device);
     cudaFree(ctx->p_stats); cudaFree(ctx->q_stats); cudaFree(ctx->p_argmax); cudaFree(ctx->status);
-    cudaFree(ctx->loop_iter); cudaFree(ctx->loop_arrived);
+    cudaFree(ctx->loop_arrived);
     if (ctx->loop_stream) cudaStreamDestroy(ctx->loop_stream);
     if (ctx->prof_start) {
         for (int k = 0; k < kProfilePairs; ++k) {
@@ -1083,8 +1084,8 @@ int svip_graph_loop_begin(svip_ctx* ctx, void* stream, const int32_t* n_active, 
     if (!ctx || !n_active || !body_stream || max_iters < 1) return SVIP_ERR_INVALID_ARG;
     if (!ctx->capturing || ctx->loop_open) return SVIP_ERR_STATE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // the iteration counter starts at zero at every replay
-    cudaError_t e = cudaMemsetAsync(ctx->loop_iter, 0, sizeof(int), st);
+    // both counters start at zero at every replay, whatever the one before has left
+    cudaError_t e = cudaMemsetAsync(ctx->loop_arrived, 0, kLoopStateBytes, st);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
     cudaGraph_t graph = nullptr;

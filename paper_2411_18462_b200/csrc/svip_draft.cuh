@@ -333,9 +333,26 @@ __device__ __forceinline__ bool drafting_done(const AdvanceArgs& a, int i, int l
     return a.policy == SVIP_POLICY_ENTROPY ? stopped || len >= a.K_cap : len >= min(a.gamma[i], a.K_cap);
 }
 
+// What the arrival that makes the counter `sum` (sequences counted in the low word, of them still drafting in the high one)
+// means for a batch of B: it closes the iteration if it is the last one.  A counter that runs past the batch holds arrivals
+// of another replay of the context's loop: the iteration is closed and the loop ended (nobody goes on), since the counts
+// mean nothing any more and a loop that nobody decides would not end.
+struct LoopArrival {
+    bool closes, overrun;
+    int going;
+};
+__host__ __device__ __forceinline__ LoopArrival loop_arrival(unsigned long long sum, int B) {
+    const unsigned n = static_cast<unsigned>(sum);
+    LoopArrival r;
+    r.closes = n >= static_cast<unsigned>(B);
+    r.overrun = n > static_cast<unsigned>(B);
+    r.going = r.overrun ? 0 : static_cast<int>(sum >> 32);
+    return r;
+}
+
 // The policy step of one sequence, taken by the draft kernel that drafted its token (one thread per sequence, those
 // that have stopped included).  The last one to arrive knows how many sequences go on and decides the loop.
-__device__ __forceinline__ void advance_one(const AdvanceArgs& a, int i, bool drafted, int len, bool stopped) {
+__device__ __forceinline__ void advance_one(const AdvanceArgs& a, int i, bool drafted, int len, bool stopped, unsigned* status) {
     bool going = false;
     if (drafted) {
         going = !drafting_done(a, i, len, stopped);
@@ -343,12 +360,12 @@ __device__ __forceinline__ void advance_one(const AdvanceArgs& a, int i, bool dr
         if (!going) a.active[i] = 0;
     }
     const unsigned long long mine = 1ull + (going ? 1ull << 32 : 0ull);
-    const unsigned long long sum = atomicAdd(a.arrived, mine) + mine;
-    if (static_cast<unsigned>(sum) == static_cast<unsigned>(a.B)) {
-        *a.arrived = 0;
-        const int n = static_cast<int>(sum >> 32);
-        *a.n_active = n;
-        loop_decide(a.loop, n);
+    const LoopArrival r = loop_arrival(atomicAdd(a.arrived, mine) + mine, a.B);
+    if (r.closes) {
+        atomicExch(a.arrived, 0ull);
+        if (r.overrun) atomicOr(status, SVIP_STATUS_LOOP_OVERLAP);
+        *a.n_active = r.going;
+        loop_decide(a.loop, r.going);
     }
 }
 
@@ -457,7 +474,7 @@ __device__ __forceinline__ void draft_row(const DraftArgs& a, int S, int rank, i
             if (a.row_stats) { a.row_stats[2 * slot] = r.m; a.row_stats[2 * slot + 1] = r.Z; }
             if (kGreedy || !ok) a.token[slot] = ((r.idx >= 0 && r.idx < a.V) ? r.idx : 0) + a.token_offset;
             // every warp of the cluster has read the position and the flag: their entries are here
-            if (kPos && a.adv.arrived) advance_one(a.adv, row, true, static_cast<int>(p) + 1, __fsqrt_rn(H) > a.thresh);
+            if (kPos && a.adv.arrived) advance_one(a.adv, row, true, static_cast<int>(p) + 1, __fsqrt_rn(H) > a.thresh, a.status);
         }
     }
     if (kGreedy) return;    // warp 0 has seen all entries land, so the block may leave
@@ -511,7 +528,7 @@ __global__ void __launch_bounds__(kThreads, kBlocks) draft_step_kernel(DraftArgs
     pdl_wait();
     if (a.active && !a.active[row]) {          // the whole cluster leaves together
         if (S > 1) cluster_wait();
-        if (kPos && a.adv.arrived && rank == 0 && tid == 0) advance_one(a.adv, row, false, 0, false);
+        if (kPos && a.adv.arrived && rank == 0 && tid == 0) advance_one(a.adv, row, false, 0, false, a.status);
         return;
     }
     long p = 0;
