@@ -248,6 +248,12 @@ int threshold_sample_den(long rows, int V, int dtype) {
     return bytes > (48L << 20) ? 2 : 1;
 }
 
+template <bool kDraft>
+auto threshold_kernel(svip_dtype dtype, const ThresholdArgs& a) -> void (*)(ThresholdArgs) {
+    if (a.top_k > 0) return dtype == SVIP_BF16 ? row_threshold_kernel<kBF16, kDraft, true> : row_threshold_kernel<kF32, kDraft, true>;
+    return dtype == SVIP_BF16 ? row_threshold_kernel<kBF16, kDraft, false> : row_threshold_kernel<kF32, kDraft, false>;
+}
+
 // The node that a stream under capture has recorded last, if its next one would depend on that one alone.
 cudaGraphNode_t last_node(cudaStream_t st) {
     cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
@@ -330,8 +336,10 @@ int svip_create(svip_ctx** out, int device, int max_rows) {
             (const void*)row_stats_kernel<kF32, 0>,      (const void*)row_stats_kernel<kF32, 1>,
             (const void*)verify_finish_kernel<kBF16>,    (const void*)verify_finish_kernel<kF32>,
             (const void*)row_stats_kernel<kBF16, 2>,     (const void*)row_stats_kernel<kF32, 2>,
-            (const void*)row_threshold_kernel<kBF16>,    (const void*)row_threshold_kernel<kF32>,
-            (const void*)row_threshold_kernel<kBF16, true>, (const void*)row_threshold_kernel<kF32, true>,
+            (const void*)row_threshold_kernel<kBF16, false, false>, (const void*)row_threshold_kernel<kF32, false, false>,
+            (const void*)row_threshold_kernel<kBF16, false, true>,  (const void*)row_threshold_kernel<kF32, false, true>,
+            (const void*)row_threshold_kernel<kBF16, true, false>,  (const void*)row_threshold_kernel<kF32, true, false>,
+            (const void*)row_threshold_kernel<kBF16, true, true>,   (const void*)row_threshold_kernel<kF32, true, true>,
             (const void*)draft_step_kernel<kBF16, false, 2, false, true>, (const void*)draft_step_kernel<kF32, false, 2, false, true>,
             (const void*)row_stats_kernel<kBF16, 1, true>, (const void*)row_stats_kernel<kF32, 1, true>,
             (const void*)verify_finish_kernel<kBF16, true>, (const void*)verify_finish_kernel<kF32, true>,
@@ -354,7 +362,7 @@ int svip_create(svip_ctx** out, int device, int max_rows) {
         attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
-        if (cudaOccupancyMaxActiveClusters(&c->max_clusters[S], (const void*)row_threshold_kernel<kF32, true>, &cfg) != cudaSuccess)
+        if (cudaOccupancyMaxActiveClusters(&c->max_clusters[S], (const void*)row_threshold_kernel<kF32, true, true>, &cfg) != cudaSuccess)
             rc = SVIP_ERR_CUDA;
     }
     if (rc == SVIP_OK) {
@@ -534,8 +542,7 @@ int svip_row_threshold(svip_ctx* ctx, const void* logits, svip_dtype dtype, int 
     a.sample_den = threshold_sample_den(n_rows, V, dtype);
     const int S = pick_threshold_cluster(ctx, n_rows, V, dtype, a.top_k > 0);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cudaError_t e = dtype == SVIP_BF16 ? launch_clustered(row_threshold_kernel<kBF16>, n_rows, S, a, st, kRingBytes)
-                                       : launch_clustered(row_threshold_kernel<kF32>, n_rows, S, a, st, kRingBytes);
+    cudaError_t e = launch_clustered(threshold_kernel<false>(dtype, a), n_rows, S, a, st, kRingBytes);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     ctx->launches += 1;
     return SVIP_OK;
@@ -563,9 +570,7 @@ int svip_draft_step_truncated(svip_ctx* ctx, const void* logits, svip_dtype dtyp
     a.sample_den = threshold_sample_den(B, V, dtype);
     const int S = pick_threshold_cluster(ctx, B, V, dtype, a.top_k > 0);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cudaError_t e = dtype == SVIP_BF16
-        ? launch_clustered(row_threshold_kernel<kBF16, true>, B, S, a, st, kRingBytes)
-        : launch_clustered(row_threshold_kernel<kF32, true>, B, S, a, st, kRingBytes);
+    cudaError_t e = launch_clustered(threshold_kernel<true>(dtype, a), B, S, a, st, kRingBytes);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     ctx->launches += 1;
     return SVIP_OK;

@@ -127,8 +127,8 @@ struct SelectShared {
     float warp_max[kWarps];
     unsigned long long warp_above[kWarps];
     // candidate path
-    SegExchange ex;                       // nucleus alone: (m, Z) of every warp segment of the cluster
-    uint4 header[kMaxCluster];            // block 0: x = number of candidates each block collected
+    SegExchange ex;                       // nucleus alone: maximum and a lower bound of Z of every warp segment of the cluster
+    uint4 header[kMaxCluster];            // block 0: x = number of candidates each block collected, (z, y) = mass of its part
     uint4 verdict;                        // x = kVerdict..., y = key of the threshold
     unsigned long long bar_group;         // all group maxima have landed
     unsigned long long bar_pool;          // block 0: headers and candidates of all blocks have landed
@@ -392,12 +392,16 @@ __device__ __forceinline__ uint32_t pool_select(SelectShared& sh, const Candidat
 //            is a lower bound of tau_k.  With G groups about -G ln(1 - k/G) elements lie above it (G >= 2k: 1.4 k),
 //            so the groups are made as large as that allows, which keeps the exchange small.
 //   nucleus  elements of mass below (1 - top_p) Z / V weigh less than (1 - top_p) Z together, so none of them is
-//            in the nucleus; (m, Z) of the row come from the first pass as in the draft step.
+//            in the nucleus, and neither with anything below Z in its place: the first pass takes maxima only, and the
+//            masses of the threads' maxima stand for Z.  The second pass also sums the masses of all elements, in fixed
+//            point and relative to the row's maximum, as the radix descent does: a cut must not depend on how many
+//            blocks share the row, nor on which way the row goes (with Z summed in fp32 it did, for running masses within
+//            1e-6 of top_p).
 // A segment that fits the ring (small launches) is still in shared memory for the second pass.  The blocks push
 // their candidates into block 0 of the cluster, which sorts up to kSortedPool of them by counting (several threads
 // per candidate), finds tau_k, the nucleus cut and the sample by scans of one warp over the sorted masses, and
 // tells the other blocks whether they are needed again.  Larger sets take radix descents in shared memory.  All
-// masses are 2^-40 fixed point, so nothing depends on the order in which candidates arrive.
+// masses are 2^-40 fixed point, so nothing depends on the order in which they are added or candidates arrive.
 // Bound by the chain of exchanges for launches of up to about 100 rows, by the two passes over the row above that.
 // Rows of 152064 bf16, top-k 50 + top-p 0.9, against cluster barriers with remote reads and a counting finish in every
 // block: draft step of 16 rows 18.3 -> 10.1 us, 64 rows 21.5 -> 14.3, 256 rows 41.0 -> 25.1; threshold of 2304 rows
@@ -465,8 +469,8 @@ __device__ __forceinline__ unsigned long long nucleus_target(float top_p, unsign
 // Block 0, warp 0: threshold, statistics and (kDraft) the sample from n <= kSortedPool candidates, sorted both ways
 // in `ps`.  Lane l owns the positions [l * per, (l + 1) * per) of both orders.  row_mass: mass of the whole row
 // (nucleus alone).  `finite` is false for a row whose maximum is not a number the masses can be taken against.
-template <bool kDraft>
-__device__ __forceinline__ void finish_sorted(const PoolScratch& ps, int n, const ThresholdArgs& a, bool use_k, bool use_p,
+template <bool kDraft, bool kTopK>
+__device__ __forceinline__ void finish_sorted(const PoolScratch& ps, int n, const ThresholdArgs& a, bool use_p,
                                               unsigned long long row_mass, float row_max, float M, bool finite, int row,
                                               int lane) {
     const int per = (n + 31) / 32;
@@ -474,10 +478,10 @@ __device__ __forceinline__ void finish_sorted(const PoolScratch& ps, int n, cons
     unsigned long long sum = 0;
     for (int i = lo; i < hi; ++i) sum += ps.mass_desc[i];
     const unsigned long long before = warp_scan_mass(sum, lane) - sum;
-    uint32_t key_t = use_k ? ps.key_desc[a.top_k - 1] : 0u;
+    uint32_t key_t = kTopK ? ps.key_desc[a.top_k - 1] : 0u;
     if (use_p && finite) {
         unsigned long long zk = row_mass;
-        if (use_k) {      // mass of the candidates >= tau_k
+        if (kTopK) {      // mass of the candidates >= tau_k
             zk = 0;
             for (int i = lo; i < hi; ++i)
                 if (ps.key_desc[i] >= key_t) zk += ps.mass_desc[i];
@@ -537,9 +541,9 @@ __device__ __forceinline__ void finish_sorted(const PoolScratch& ps, int n, cons
 // Block 0 with all candidates of the cluster in ps.pool: finds the threshold and writes what it can.  Returns the
 // verdict for the row (kVerdictDone, or kVerdictStream when the draft step has to be streamed at key_out), which
 // `tell` passes on to the other blocks as soon as it is certain.
-template <int DT, bool kDraft, class Tell>
-__device__ __forceinline__ uint32_t finish_pool(SelectShared& sh, PoolScratch& ps, int n, const ThresholdArgs& a,
-                                                bool use_k, bool use_p, unsigned long long row_mass, int row, int tid,
+template <int DT, bool kDraft, bool kTopK, class Tell>
+__device__ __forceinline__ uint32_t finish_pool(SelectShared& sh, PoolScratch& ps, int n, const ThresholdArgs& a, bool use_p,
+                                                unsigned long long row_mass, int row, int tid,
                                                 uint32_t& key_out, Tell&& tell) {
     constexpr int kLevels = DT == kBF16 ? 2 : 4;
     const int lane = tid & 31, warp = tid >> 5;
@@ -573,16 +577,16 @@ __device__ __forceinline__ uint32_t finish_pool(SelectShared& sh, PoolScratch& p
             ps.mass_idx[left] = w;
         }
         __syncthreads();
-        key_out = use_k ? ps.key_desc[a.top_k - 1] : 0u;   // what a row without finite mass is cut at
+        key_out = kTopK ? ps.key_desc[a.top_k - 1] : 0u;   // what a row without finite mass is cut at
         tell(verdict, key_out);
         if (verdict == kVerdictStream) {
             if (tid == 0) a.thr[row] = key_out ? key_value(key_out) : neg_inf();
         } else if (warp == 0) {
-            finish_sorted<kDraft>(ps, n, a, use_k, use_p, row_mass, row_max, M, finite, row, lane);
+            finish_sorted<kDraft, kTopK>(ps, n, a, use_p, row_mass, row_max, M, finite, row, lane);
         }
         return verdict;
     }
-    uint32_t key_t = use_k ? pool_select<kLevels, false>(sh, ps.pool, n, static_cast<uint32_t>(a.top_k), 0ull, 0.f, 0.f, tid) : 0u;
+    uint32_t key_t = kTopK ? pool_select<kLevels, false>(sh, ps.pool, n, static_cast<uint32_t>(a.top_k), 0ull, 0.f, 0.f, tid) : 0u;
     uint32_t top = 0;
     if (tid == 0) sh.top_key = 0;
     __syncthreads();
@@ -600,9 +604,9 @@ __device__ __forceinline__ uint32_t finish_pool(SelectShared& sh, PoolScratch& p
         return block_sum_u64(sh, z, tid);
     };
     if (use_p && finite) {
-        const unsigned long long zk = use_k ? mass_from(key_t) : row_mass;
+        const unsigned long long zk = kTopK ? mass_from(key_t) : row_mass;
         if (zk > 0) {
-            const unsigned long long all = use_k ? zk : mass_from(0u);
+            const unsigned long long all = kTopK ? zk : mass_from(0u);
             unsigned long long want = nucleus_target(a.top_p, zk);
             if (want > all) want = all;                // rounding at the very end of the candidates: all of them
             key_t = max(key_t, pool_select<kLevels, true>(sh, ps.pool, n, 0u, want, a.c, M, tid));
@@ -622,22 +626,68 @@ __device__ __forceinline__ uint32_t finish_pool(SelectShared& sh, PoolScratch& p
     return kVerdictDone;
 }
 
-// Collects the elements >= t0v of the block's segments into sh.cand.  `resident`: every segment of the row fits the
-// ring and lies there since pass 1 (a property of the row, so the same in every warp: a block barrier depends on it).
+// Sum of the 2^-40 fixed-point masses of elements of a row (those of mass_of_key).  Bound by instructions: nearly all elements
+// weigh less than 2^-17, and for these the addition of 2^23 rounded towards zero leaves the integer in the mantissa, two
+// elements per instruction on the wide pipe, where a conversion takes the pipe of the exponentials.  A vector with a
+// likelier element, or with a NaN (which shows as a sum that no EPV masses have), converts.  Round of 64 sequences with top-p
+// 0.95 (5 draft steps, thresholds of 384 rows of 304 KB): 144 us; one element at a time and in one kernel with the top-k
+// 173; with the total summed in fp32 in the first pass, in whatever order the launch shape gave, 141.
 template <int DT>
+struct MassSum {
+    float c, M;
+    float big;                    // no element below this logit weighs 2^-17 or more
+    unsigned long long sum = 0;
+    __device__ __forceinline__ MassSum(float c_, float row_max) {
+        c = c_;
+        M = __fmul_rn(row_max, c_);
+        big = (M - 17.01f) / c - 5e-7f * fabsf(row_max);
+    }
+    __device__ __forceinline__ void one(float x) {
+        sum += __float2ull_rz(ex2_approx(fmaxf(__fmaf_rn(x, c, -M), kArgFloor)) * kMassScale);
+    }
+    __device__ __forceinline__ void vector(const uint4& raw, float vmax) {
+        constexpr int EPV = ElemTraits<DT>::kEPV;
+        float x[EPV];
+        ElemTraits<DT>::unpack(raw, x);
+        const f32x2 c2 = pack2(c, c), nm2 = pack2(-M, -M), scale2 = pack2(kMassScale, kMassScale), base2 = pack2(8388608.f, 8388608.f);
+        uint32_t s = 0;
+#pragma unroll
+        for (int j = 0; j < EPV; j += 2) {
+            float a0, a1;
+            unpack2(fma2(pack2(x[j], x[j + 1]), c2, nm2), a0, a1);
+            unpack2(fma2_rz(pack2(ex2_approx(a0), ex2_approx(a1)), scale2, base2), a0, a1);
+            s += __float_as_uint(a0) + __float_as_uint(a1);
+        }
+        s -= EPV * 0x4B000000u;               // EPV masses below 2^23
+        if (vmax >= big || s >= EPV * (1u << 23)) {
+#pragma unroll
+            for (int j = 0; j < EPV; ++j) one(x[j]);
+        } else {
+            sum += s;
+        }
+    }
+};
+
+// Collects the elements >= t0v of the block's segments into sh.cand and (kMass) leaves the mass of all elements of every
+// warp's segment in sh.warp_above.  `resident`: every segment of the row fits the ring and lies there since pass 1 (a
+// property of the row, so the same in every warp: a block barrier depends on it).
+template <int DT, bool kMass>
 __device__ __forceinline__ void collect(const RowGeom& g, const LaneSpan& s, bool resident, uint32_t slot0, float t0v,
-                                        uint32_t cap, SelectShared& sh) {
+                                        uint32_t cap, SelectShared& sh, float c, float row_max) {
     constexpr int EPV = ElemTraits<DT>::kEPV;
+    MassSum<DT> mass(c, row_max);
     const bool lowest = !(t0v > neg_inf());      // no bound: every element, -inf and NaN (which counts as -inf) among them
     auto take = [&](float x, int i) {
         const uint32_t pos = atomicAdd(&sh.n_cand, 1u);
         if (pos < cap) sh.cand[pos] = Candidate{order_key(x), static_cast<uint32_t>(i)};
     };
-    auto has = [&](const uint4& raw) {
+    auto has = [&](const uint4& raw) {        // asked once per vector: it also counts its mass
         RawMax<DT> m;
         m.reset();
         m.fold(raw);
-        return m.value() >= t0v || lowest;
+        const float top = m.value();
+        if (kMass) mass.vector(raw, top);
+        return top >= t0v || lowest;
     };
     auto visit = [&](const uint4& raw, int vi) {
         float x[EPV];
@@ -652,7 +702,9 @@ __device__ __forceinline__ void collect(const RowGeom& g, const LaneSpan& s, boo
 #pragma unroll
         for (int j = 0; j < EPV; ++j) {
             const int i = vi * EPV + j - g.pre;
-            if (i >= 0 && i < g.V && (x[j] >= t0v || lowest)) take(x[j], i);
+            if (i < 0 || i >= g.V) continue;
+            if (kMass) mass.one(x[j]);
+            if (x[j] >= t0v || lowest) take(x[j], i);
         }
     };
     if (resident) {
@@ -678,6 +730,10 @@ __device__ __forceinline__ void collect(const RowGeom& g, const LaneSpan& s, boo
     }
     if (s.head) edge(0);
     if (s.tail) edge(g.nvec - 1);
+    if (kMass) {
+        const unsigned long long m = warp_scan_mass(mass.sum, threadIdx.x & 31);
+        if ((threadIdx.x & 31) == 31) sh.warp_above[threadIdx.x >> 5] = m;
+    }
 }
 
 // Groups of threads per warp whose maxima bound a top-k: a power of two, at least 2 k in the cluster if there are
@@ -709,9 +765,9 @@ __device__ __forceinline__ void candidate_open(SelectShared& sh, int S, int rank
 
 // The whole path for one row, opened by candidate_open(); the same verdict in every block of the cluster.  For the
 // nucleus alone row_max receives the largest logit of the row.
-template <int DT, bool kDraft>
+template <int DT, bool kDraft, bool kTopK>
 __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneSpan& span, int S, int rank, int tid,
-                                                   uint32_t slot0, const ThresholdArgs& a, bool use_k, bool use_p, int row,
+                                                   uint32_t slot0, const ThresholdArgs& a, bool use_p, int row,
                                                    SelectShared& sh, PoolScratch* scratch, uint32_t& key_out, float& row_max) {
     constexpr int EPV = ElemTraits<DT>::kEPV;
     const int lane = tid & 31, warp = tid >> 5;
@@ -719,22 +775,21 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
     const uint32_t cap = static_cast<uint32_t>(S == 1 ? kCandPerBlock : min(kCandPerBlock, kPoolCap / S));
     const int gs = group_shift(S, a.top_k);
     const int n_groups = (kWarps * S) << gs;
-    unsigned long long row_mass = 0;
     uint32_t parity = 0;
-    int den = use_k ? a.sample_den : 1;
+    int den = kTopK ? a.sample_den : 1;
     for (;;) {
-        // ---- pass 1: the bound
-        if (use_k) {
-            const LaneSpan part = den > 1 ? lane_span<DT>(g, seg, lane, den) : span;
-            RawMax<DT> m;
-            m.reset();
-            stream_interior(part, slot0, [&](const uint4& raw, int) { m.fold(raw); });
-            float best = m.value();
-            if (part.head || part.tail) {
-                float x[EPV];
-                if (part.head) { unpack_masked<DT>(ld_vec(g.base), 0, g, x); best = fmaxf(best, vec_max<EPV>(x)); }
-                if (part.tail) { unpack_masked<DT>(ld_vec(g.base + g.nvec - 1), g.nvec - 1, g, x); best = fmaxf(best, vec_max<EPV>(x)); }
-            }
+        // ---- pass 1: the largest logit of every thread, and from these the bound
+        const LaneSpan part = den > 1 ? lane_span<DT>(g, seg, lane, den) : span;
+        RawMax<DT> m;
+        m.reset();
+        stream_interior(part, slot0, [&](const uint4& raw, int) { m.fold(raw); });
+        float best = m.value();
+        if (part.head || part.tail) {
+            float x[EPV];
+            if (part.head) { unpack_masked<DT>(ld_vec(g.base), 0, g, x); best = fmaxf(best, vec_max<EPV>(x)); }
+            if (part.tail) { unpack_masked<DT>(ld_vec(g.base + g.nvec - 1), g.nvec - 1, g, x); best = fmaxf(best, vec_max<EPV>(x)); }
+        }
+        if constexpr (kTopK) {
             const int width = 32 >> gs;
             for (int o = width >> 1; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
             const int slot = (seg << gs) + (lane >> (5 - gs));
@@ -753,7 +808,9 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
             }
             kth_largest(sh, n_groups, static_cast<uint32_t>(a.top_k), tid);
         } else {
-            const Partial t = reduce_segment<DT, 1, false>(g, span, seg, a.c, lane, slot0, neg_inf());
+            Partial t;
+            t.m = warp_max(best); t.idx = kIntMax; t.A = 0.f;
+            t.Z = warp_sum(best > neg_inf() ? ex2_approx(fmaxf((best - t.m) * a.c, kArgFloor)) : 0.f);
             if (S == 1) {
                 if (lane == 0) { SegEntry& e = sh.ex.all[warp]; e.m = t.m; e.idx = t.idx; e.Z = t.Z; e.A = 0.f; }
                 __syncthreads();
@@ -768,7 +825,6 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
             if (!(fabsf(r.m) <= kMaxLogit) || !(r.Z > 0.f)) return kVerdictDescend;   // in every block alike
             // no element weighs more than 1, so the nucleus has at least top_p Z of them: a flat row does not fit
             if (a.top_p * r.Z > static_cast<float>(kPoolCap)) return kVerdictDescend;
-            row_mass = static_cast<unsigned long long>(static_cast<double>(r.Z) * static_cast<double>(kMassScale));
             // in log2 units, a little low for the roundings of the weights, and of the bound as a logit
             const float cut = log2f((1.f - a.top_p) * r.Z / static_cast<float>(g.V)) - 0.05f;
             if (tid == 0) sh.bound_key = order_key((__fmul_rn(r.m, a.c) + cut) / a.c - 5e-7f * fabsf(r.m));
@@ -777,17 +833,24 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
         // ---- pass 2: the candidates
         const float t0v = key_value(sh.bound_key);
         pdl_launch_dependents();
-        collect<DT>(g, span, den == 1 && g.vps <= 32 * kStages, slot0, t0v, cap, sh);
+        const bool resident = den == 1 && g.vps <= 32 * kStages;
+        collect<DT, !kTopK>(g, span, resident, slot0, t0v, cap, sh, a.c, row_max);
         __syncthreads();
         uint32_t verdict;
         const uint32_t mine = sh.n_cand;
+        unsigned long long my_mass = 0;
+        if (!kTopK) {
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) my_mass += sh.warp_above[w];
+        }
         if (S > 1 && rank != 0) {
             const uint32_t sent = mine <= cap ? mine : 0u;
             const uint32_t bar0 = map_to_rank(smem_addr(&sh.bar_pool), 0);
             for (uint32_t i = tid; i < sent; i += kThreads)
                 push8(map_to_rank(smem_addr(&sh.landing[rank * cap + i]), 0), bar0, sh.cand[i].key, sh.cand[i].idx);
             if (tid == 0) {
-                push16(map_to_rank(smem_addr(&sh.header[rank]), 0), bar0, mine, 0u, 0u, 0u);
+                push16(map_to_rank(smem_addr(&sh.header[rank]), 0), bar0, mine, static_cast<uint32_t>(my_mass),
+                       static_cast<uint32_t>(my_mass >> 32), 0u);
                 mbar_arrive_expect_tx_remote(bar0, 16u + 8u * sent);
             }
             bar_wait(sh.bar_verdict, parity, a.status, tid);
@@ -795,10 +858,7 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
             key_out = sh.verdict.y;
         } else {
             if (S > 1) {
-                if (tid == 0) {
-                    sh.header[0] = make_uint4(mine, 0u, 0u, 0u);
-                    mbar_arrive_expect_tx(smem_addr(&sh.bar_pool), 0);
-                }
+                if (tid == 0) mbar_arrive_expect_tx(smem_addr(&sh.bar_pool), 0);
                 bar_wait(sh.bar_pool, parity, a.status, tid);
             }
             // tells the other blocks, once
@@ -807,7 +867,10 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
                     push16(map_to_rank(smem_addr(&sh.verdict), tid), map_to_rank(smem_addr(&sh.bar_verdict), tid), v, key, 0u, 0u);
             };
             // lane r holds the count of block r; every warp knows all offsets
-            const uint32_t count = lane == 0 ? mine : lane < S ? sh.header[lane].x : 0u;
+            const uint4 head = lane > 0 && lane < S ? sh.header[lane] : make_uint4(0u, 0u, 0u, 0u);
+            const uint32_t count = lane == 0 ? mine : head.x;
+            unsigned long long row_mass = 0;
+            if (!kTopK) row_mass = shfl_u64(warp_scan_mass((static_cast<unsigned long long>(head.z) << 32) | head.y, lane), 31) + my_mass;
             const bool fits = !__any_sync(0xffffffffu, count > cap);
             uint32_t end = count;
 #pragma unroll
@@ -816,7 +879,7 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
                 if (lane >= o) end += up;
             }
             const uint32_t total = __shfl_sync(0xffffffffu, end, kMaxCluster - 1);
-            if (!fits || total < static_cast<uint32_t>(use_k ? a.top_k : 1)) {
+            if (!fits || total < static_cast<uint32_t>(kTopK ? a.top_k : 1)) {
                 verdict = !fits && den > 1 ? kVerdictRetry : kVerdictDescend;
                 tell(verdict, 0u);
             } else {
@@ -826,7 +889,7 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
                 const Candidate* from = r == 0 ? sh.cand : sh.landing + r * cap;
                 for (uint32_t t = (warp / kMaxCluster) * 32 + lane; t < nr; t += 64) scratch->pool[to + t] = from[t];
                 __syncthreads();
-                verdict = finish_pool<DT, kDraft>(sh, *scratch, static_cast<int>(total), a, use_k, use_p, row_mass, row, tid,
+                verdict = finish_pool<DT, kDraft, kTopK>(sh, *scratch, static_cast<int>(total), a, use_p, row_mass, row, tid,
                                                   key_out, tell);
             }
         }
@@ -866,8 +929,9 @@ __device__ __forceinline__ void draft_at_threshold(const ThresholdArgs& a, int S
 }
 
 // kDraft: the truncated draft step in the same launch: from the candidates where that path applies,
-// else by streaming the row once more at the threshold just found.
-template <int DT, bool kDraft = false>
+// else by streaming the row once more at the threshold just found.  kTopK: with a top_k in [1, V), else the nucleus alone (or
+// nothing at all); two kernels rather than one, whose registers did not suffice for both.
+template <int DT, bool kDraft, bool kTopK>
 __global__ void __launch_bounds__(kThreads, 2) row_threshold_kernel(ThresholdArgs a) {
     constexpr int kLevels = DT == kBF16 ? 2 : 4;   // the low 16 bits of a bf16 logit carry nothing
     extern __shared__ __align__(kRingAlign) uint4 ring[];
@@ -881,12 +945,11 @@ __global__ void __launch_bounds__(kThreads, 2) row_threshold_kernel(ThresholdArg
                      static_cast<size_t>(row) * a.row_stride * ElemTraits<DT>::kBytes;
     const RowGeom g = make_geom<DT>(rp, a.V, S * kWarps);
     const uint32_t slot0 = static_cast<uint32_t>(__cvta_generic_to_shared(ring)) + tid * 16;
-    const bool use_k = a.top_k >= 1 && a.top_k < a.V;
     const bool use_p = a.top_p < 1.0f;
     // a small k against the number of threads of the cluster, or the nucleus alone: two passes over the row
-    const bool by_candidates = use_k ? a.top_k <= (S * kThreads) / 4 : use_p;
+    const bool by_candidates = kTopK ? a.top_k <= (S * kThreads) / 4 : use_p;
     const LaneSpan span = lane_span<DT>(g, rank * kWarps + warp, lane);
-    if (by_candidates) candidate_open(sh, S, rank, a.top_k, use_k, tid);
+    if (by_candidates) candidate_open(sh, S, rank, a.top_k, kTopK, tid);
     if (!a.active && lane == 0) prefetch_segment(g, rank * kWarps + warp, kRingBytes / kWarps);
     pdl_wait();
     if (kDraft && a.active && !a.active[row]) {         // the whole cluster leaves together
@@ -901,9 +964,9 @@ __global__ void __launch_bounds__(kThreads, 2) row_threshold_kernel(ThresholdArg
 
     if (by_candidates) {
         uint32_t key_t = 0;
-        const uint32_t verdict = candidate_path<DT, kDraft>(g, span, S, rank, tid, slot0, a, use_k, use_p, row, sh,
-                                                            reinterpret_cast<PoolScratch*>(ring), key_t, row_max);
-        have_max = !use_k;
+        const uint32_t verdict = candidate_path<DT, kDraft, kTopK>(g, span, S, rank, tid, slot0, a, use_p, row, sh,
+                                                                   reinterpret_cast<PoolScratch*>(ring), key_t, row_max);
+        have_max = !kTopK;
         if (verdict == kVerdictDone) return;
         if (kDraft && verdict == kVerdictStream) {
             __syncthreads();       // block 0 is done with the ring in every warp
@@ -912,7 +975,7 @@ __global__ void __launch_bounds__(kThreads, 2) row_threshold_kernel(ThresholdArg
         }
     }
 
-    if (use_k) {
+    if (kTopK) {
         uint32_t prefix = 0, k_rem = static_cast<uint32_t>(a.top_k);
         for (int level = 0; level < kLevels; ++level) {
             const int shift = 24 - 8 * level;
