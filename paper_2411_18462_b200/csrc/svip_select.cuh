@@ -27,7 +27,7 @@ constexpr int kHistCopies = 8;           // interleaved copies of the histogram:
 constexpr float kMassScale = 1099511627776.0f;   // 2^40
 constexpr int kPoolCap = 2048;           // candidates of the whole cluster
 constexpr int kCandPerBlock = 1024;      // candidates one block may collect (less when blocks share the pool)
-constexpr int kSortedPool = 512;         // up to this many candidates are finished by sorting them
+constexpr int kCounted = 256;            // up to this many group maxima or candidates are put in order by counting
 constexpr int kMaxGroups = 2048;         // groups of threads whose maxima give the bound of a top-k
 
 struct ThresholdArgs {
@@ -101,7 +101,7 @@ enum : uint32_t {
     kVerdictDone = 0,     // block 0 writes every output
     kVerdictDescend = 1,  // the candidates do not fit: radix descent over the row
     kVerdictRetry = 2,    // the same after a bound from part of the row: once more with the bound from all of it
-    kVerdictStream = 3    // the threshold is known, the draft step streams the row once more at it
+    kVerdictStream = 3    // a row without finite mass: the draft step streams it once more at the threshold
 };
 
 struct SelectShared {
@@ -148,10 +148,15 @@ struct SelectShared {
 // Block 0's working set while it finishes a row from its candidates; lives in the streaming ring, free by then.
 struct PoolScratch {
     Candidate pool[kPoolCap];
-    uint32_t key_desc[kSortedPool];                  // keys from the largest down ...
-    unsigned long long mass_desc[kSortedPool];       // ... and their masses
-    Candidate by_idx[kSortedPool];                   // candidates in index order ...
-    unsigned long long mass_idx[kSortedPool];        // ... and their masses
+    union {
+        struct {                                         // up to kCounted candidates
+            uint32_t key_desc[kCounted];                 // keys from the largest down ...
+            unsigned long long mass_desc[kCounted];      // ... and their masses
+            Candidate by_idx[kCounted];                  // candidates in index order ...
+            unsigned long long mass_idx[kCounted];       // ... and their masses
+        };
+        unsigned long long mass[kPoolCap];               // more: the masses of the pool
+    };
 };
 static_assert(sizeof(PoolScratch) <= kRingBytes, "the pool is finished inside the ring");
 
@@ -159,6 +164,15 @@ __device__ __forceinline__ unsigned long long shfl_up_u64(unsigned long long v, 
     uint32_t lo = __shfl_up_sync(0xffffffffu, static_cast<uint32_t>(v), o);
     uint32_t hi = __shfl_up_sync(0xffffffffu, static_cast<uint32_t>(v >> 32), o);
     return (static_cast<unsigned long long>(hi) << 32) | lo;
+}
+
+// Adds a mass to a bin of the interleaved histogram copies of the calling lane, as two 32-bit words with carry (64-bit atomics
+// on shared memory are loops, which crawl where many candidates share a bin).
+__device__ __forceinline__ void add_mass(uint32_t* h_lo, uint32_t* h_hi, uint32_t bin, unsigned long long w) {
+    const uint32_t lo = static_cast<uint32_t>(w);
+    const uint32_t old = atomicAdd(h_lo + bin * kHistCopies, lo);
+    const uint32_t hi = static_cast<uint32_t>(w >> 32) + (old + lo < old ? 1u : 0u);
+    if (hi) atomicAdd(h_hi + bin * kHistCopies, hi);
 }
 
 // One pass: histogram of digit (key >> shift) & 255 over the elements whose higher digits equal
@@ -193,16 +207,9 @@ __device__ __forceinline__ void histogram_pass(cg::cluster_group& cluster, const
             }
             // the nucleus descent is decided by the masses alone, the top-k descent by the counts
             if ((first || (key >> (shift + 8)) == want) && (!kMass || wq)) {
-                const uint32_t bin = ((key >> shift) & 255u) * kHistCopies;
-                if (!kMass) {
-                    atomicAdd(h_cnt + bin, 1u);
-                } else {
-                    const uint32_t lo = static_cast<uint32_t>(wq);
-                    const uint32_t old = atomicAdd(h_lo + bin, lo);
-                    const uint32_t carry = (old + lo < old) ? 1u : 0u;
-                    const uint32_t hi = static_cast<uint32_t>(wq >> 32) + carry;
-                    if (hi) atomicAdd(h_hi + bin, hi);
-                }
+                const uint32_t bin = (key >> shift) & 255u;
+                if (!kMass) atomicAdd(h_cnt + bin * kHistCopies, 1u);
+                else add_mass(h_lo, h_hi, bin, wq);
             }
         }
     });
@@ -320,21 +327,32 @@ __device__ __forceinline__ void decide(SelectShared& sh, int lane, uint32_t k_re
     }
 }
 
-// Sum of one 64-bit integer per thread over the block (every thread gets it).  Two barriers.
-__device__ __forceinline__ unsigned long long block_sum_u64(SelectShared& sh, unsigned long long v, int tid) {
-    const int lane = tid & 31, warp = tid >> 5;
+// Inclusive prefix over the lanes of per-lane masses.
+__device__ __forceinline__ unsigned long long warp_scan_mass(unsigned long long v, int lane) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        uint32_t lo = __shfl_xor_sync(0xffffffffu, static_cast<uint32_t>(v), o);
-        uint32_t hi = __shfl_xor_sync(0xffffffffu, static_cast<uint32_t>(v >> 32), o);
-        v += (static_cast<unsigned long long>(hi) << 32) | lo;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long up = shfl_up_u64(v, o);
+        if (lane >= o) v += up;
     }
-    __syncthreads();   // warp_above may still be read from an earlier use
-    if (lane == 0) sh.warp_above[warp] = v;
-    __syncthreads();
-    v = 0;
-    for (int w = 0; w < kWarps; ++w) v += sh.warp_above[w];
     return v;
+}
+
+// Sum of the integers of the threads before this one, and of all of them.  Two barriers.
+__device__ __forceinline__ unsigned long long block_prefix_u64(SelectShared& sh, unsigned long long v, int tid,
+                                                               unsigned long long& total) {
+    const int lane = tid & 31, warp = tid >> 5;
+    const unsigned long long incl = warp_scan_mass(v, lane);
+    __syncthreads();   // warp_above may still be read from an earlier use
+    if (lane == 31) sh.warp_above[warp] = incl;
+    __syncthreads();
+    unsigned long long before = 0;
+    total = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+        if (w == warp) before = total;
+        total += sh.warp_above[w];
+    }
+    return before + incl - v;
 }
 
 // What the statistics output holds for a row: (m, Z~) in the convention of the draft step's row_stats.
@@ -345,42 +363,6 @@ __device__ __forceinline__ float2 kept_stats(float row_max, unsigned long long k
 __device__ __forceinline__ unsigned long long mass_of_key(uint32_t key, float c, float M) {
     const float w = ex2_approx(fmaxf(__fmaf_rn(key_value(key), c, -M), kArgFloor));
     return __float2ull_rz(w * kMassScale);
-}
-
-// Radix descent over `n` keys held in shared memory, the same in every block of the cluster, so
-// no exchange is needed: the k_rem-th largest key (by counts), or the key at which the running mass
-// from the top reaches p_rem.  Block-collective.
-template <int kLevels, bool kByMass>
-__device__ __forceinline__ uint32_t pool_select(SelectShared& sh, const Candidate* pool, int n, uint32_t k_rem,
-                                                unsigned long long p_rem, float c, float M, int tid) {
-    const int lane = tid & 31, warp = tid >> 5;
-    uint32_t prefix = 0;
-    for (int level = 0; level < kLevels; ++level) {
-        const int shift = 24 - 8 * level;
-        if (tid < 256) { sh.tot_cnt[tid] = 0; sh.tot_mass[tid] = 0; }
-        __syncthreads();
-        for (int i = tid; i < n; i += kThreads) {
-            const uint32_t key = pool[i].key;
-            if (level == 0 || (key >> (shift + 8)) == (prefix >> (shift + 8))) {
-                const uint32_t bin = (key >> shift) & 255u;
-                if (!kByMass) {
-                    atomicAdd(&sh.tot_cnt[bin], 1u);
-                } else {
-                    const unsigned long long wq = mass_of_key(key, c, M);
-                    if (wq) atomicAdd(&sh.tot_mass[bin], wq);
-                }
-            }
-        }
-        __syncthreads();
-        if (warp == 0) decide<kByMass>(sh, lane, k_rem, p_rem);
-        __syncthreads();
-        prefix |= static_cast<uint32_t>(sh.bin) << shift;
-        k_rem -= sh.cnt_above;
-        p_rem -= sh.mass_above;
-        __syncthreads();
-    }
-    if (kLevels == 2 && !(prefix & 0x80000000u)) prefix |= 0xffffu;
-    return prefix;
 }
 
 // ------------------------------------------------------------------ candidate path
@@ -398,9 +380,9 @@ __device__ __forceinline__ uint32_t pool_select(SelectShared& sh, const Candidat
 //            blocks share the row, nor on which way the row goes (with Z summed in fp32 it did, for running masses within
 //            1e-6 of top_p).
 // A segment that fits the ring (small launches) is still in shared memory for the second pass.  The blocks push
-// their candidates into block 0 of the cluster, which sorts up to kSortedPool of them by counting (several threads
-// per candidate), finds tau_k, the nucleus cut and the sample by scans of one warp over the sorted masses, and
-// tells the other blocks whether they are needed again.  Larger sets take radix descents in shared memory.  All
+// their candidates into block 0 of the cluster, which puts up to kCounted of them in order by counting (several threads
+// per candidate) and finds tau_k, the nucleus cut and the sample by scans of one warp over the masses; in more these are
+// found by radix descents in shared memory.  It tells the other blocks whether they are needed again.  All
 // masses are 2^-40 fixed point, so nothing depends on the order in which they are added or candidates arrive.
 // Bound by the chain of exchanges for launches of up to about 100 rows, by the two passes over the row above that.
 // Rows of 152064 bf16, top-k 50 + top-p 0.9, against cluster barriers with remote reads and a counting finish in every
@@ -420,9 +402,66 @@ __device__ __forceinline__ int share_shift(int n) {
     return k;
 }
 
-// Leaves the k-th largest of the n values in sh.bound_key (as an order key), by counting: it is the smallest value
-// with fewer than k values above it.  Ends with a barrier.  (n <= kMaxGroups, a multiple of 16; 1 <= k <= n.)
+// Radix descent over n items of shared memory in bits [low, high) of their keys, at most 8 bits a level; `prefix` holds the
+// bits from `high` up, which all items share.  The key of the k_rem-th item from the top (by counts), or the one at which the
+// running mass from the top reaches p_rem.  By mass the histogram copies are used, which in the candidate path are the
+// landing place of the peers' candidates.  Block-collective; ends with a barrier.
+template <bool kByMass, class KeyOf, class MassOf>
+__device__ __forceinline__ uint32_t pool_select(SelectShared& sh, int n, uint32_t prefix, int high, int low, uint32_t k_rem,
+                                                unsigned long long p_rem, int tid, const KeyOf& key_of, const MassOf& mass_of) {
+    const int lane = tid & 31, warp = tid >> 5;
+#pragma unroll 1
+    while (high > low) {
+        const int shift = max(high - 8, low);
+        const uint32_t digits = (1u << (high - shift)) - 1u;
+        if (kByMass) {
+            for (int i = tid; i < 256 * kHistCopies; i += kThreads) { (&sh.priv[1][0][0])[i] = 0; (&sh.priv[2][0][0])[i] = 0; }
+        }
+        if (tid < 256) { sh.tot_cnt[tid] = 0; sh.tot_mass[tid] = 0; }
+        __syncthreads();
+        for (int i = tid; i < n; i += kThreads) {
+            const uint32_t key = key_of(i);
+            if (high < 32 && (key >> high) != (prefix >> high)) continue;
+            const uint32_t bin = (key >> shift) & digits;
+            if (!kByMass) {
+                atomicAdd(&sh.tot_cnt[bin], 1u);
+            } else {
+                const unsigned long long w = mass_of(i);
+                if (w) add_mass(&sh.priv[1][0][lane % kHistCopies], &sh.priv[2][0][lane % kHistCopies], bin, w);
+            }
+        }
+        __syncthreads();
+        if (kByMass) {
+            if (tid < 256) {
+                unsigned long long m = 0;
+#pragma unroll
+                for (int k = 0; k < kHistCopies; ++k)
+                    m += (static_cast<unsigned long long>(sh.priv[2][tid][k]) << 32) + sh.priv[1][tid][k];
+                sh.tot_mass[tid] = m;
+            }
+            __syncthreads();
+        }
+        if (warp == 0) decide<kByMass>(sh, lane, k_rem, p_rem);
+        __syncthreads();
+        prefix |= static_cast<uint32_t>(sh.bin) << shift;
+        k_rem -= sh.cnt_above;
+        p_rem -= sh.mass_above;
+        high = shift;
+    }
+    return prefix;
+}
+
+// Leaves in sh.bound_key the k-th largest of the n values (as an order key), or somewhat less.  Few values by counting: it is
+// the smallest value with fewer than k values above it.  That is quadratic (2048 values: 190 us), so of more the upper 16 bits
+// are found by a descent and the others left zero.  Ends with a barrier.  (n <= kMaxGroups, a multiple of 16; 1 <= k <= n.)
 __device__ __forceinline__ void kth_largest(SelectShared& sh, int n, uint32_t k, int tid) {
+    if (n > kCounted) {
+        const auto key_of = [&](int i) { return order_key(sh.group_max[i]); };
+        const uint32_t key = pool_select<false>(sh, n, 0u, 32, 16, k, 0ull, tid, key_of, key_of);
+        if (tid == 0) sh.bound_key = key;
+        __syncthreads();
+        return;
+    }
     const int shift = share_shift(n), per = 1 << shift, rows = kThreads >> shift;
     const int sub = tid & (per - 1);
     const float4* quads = reinterpret_cast<const float4*>(sh.group_max);
@@ -444,15 +483,6 @@ __device__ __forceinline__ void kth_largest(SelectShared& sh, int n, uint32_t k,
     __syncthreads();
 }
 
-// Inclusive prefix over the lanes of per-lane masses.
-__device__ __forceinline__ unsigned long long warp_scan_mass(unsigned long long v, int lane) {
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long up = shfl_up_u64(v, o);
-        if (lane >= o) v += up;
-    }
-    return v;
-}
 __device__ __forceinline__ unsigned long long shfl_u64(unsigned long long v, int src) {
     const uint32_t lo = __shfl_sync(0xffffffffu, static_cast<uint32_t>(v), src);
     const uint32_t hi = __shfl_sync(0xffffffffu, static_cast<uint32_t>(v >> 32), src);
@@ -466,7 +496,7 @@ __device__ __forceinline__ unsigned long long nucleus_target(float top_p, unsign
     return want > total ? total : want;
 }
 
-// Block 0, warp 0: threshold, statistics and (kDraft) the sample from n <= kSortedPool candidates, sorted both ways
+// Block 0, warp 0: threshold, statistics and (kDraft) the sample from n <= kCounted candidates, in order both ways
 // in `ps`.  Lane l owns the positions [l * per, (l + 1) * per) of both orders.  row_mass: mass of the whole row
 // (nucleus alone).  `finite` is false for a row whose maximum is not a number the masses can be taken against.
 template <bool kDraft, bool kTopK>
@@ -545,9 +575,8 @@ template <int DT, bool kDraft, bool kTopK, class Tell>
 __device__ __forceinline__ uint32_t finish_pool(SelectShared& sh, PoolScratch& ps, int n, const ThresholdArgs& a, bool use_p,
                                                 unsigned long long row_mass, int row, int tid,
                                                 uint32_t& key_out, Tell&& tell) {
-    constexpr int kLevels = DT == kBF16 ? 2 : 4;
     const int lane = tid & 31, warp = tid >> 5;
-    if (n <= kSortedPool) {
+    if (n <= kCounted) {
         // position of every candidate in both orders, by counting; `per` threads share a candidate
         const int shift = share_shift(n), per = 1 << shift;
         const int sub = tid & (per - 1), i = tid >> shift;
@@ -586,44 +615,80 @@ __device__ __forceinline__ uint32_t finish_pool(SelectShared& sh, PoolScratch& p
         }
         return verdict;
     }
-    uint32_t key_t = kTopK ? pool_select<kLevels, false>(sh, ps.pool, n, static_cast<uint32_t>(a.top_k), 0ull, 0.f, 0.f, tid) : 0u;
-    uint32_t top = 0;
+    // a larger set: radix descents, for the threshold in the keys and for the sample in the indices
     if (tid == 0) sh.top_key = 0;
     __syncthreads();
+    uint32_t top = 0;
     for (int i = tid; i < n; i += kThreads) top = max(top, ps.pool[i].key);
     top = __reduce_max_sync(0xffffffffu, top);
     if (lane == 0) atomicMax(&sh.top_key, top);
     __syncthreads();
-    const float row_max = key_value(sh.top_key);
+    top = sh.top_key;
+    const float row_max = key_value(top);          // the largest candidate is the largest logit of the row
     const bool finite = fabsf(row_max) <= kMaxLogit;
     const float M = finite ? __fmul_rn(row_max, a.c) : 0.f;
-    auto mass_from = [&](uint32_t key) {
+    const uint32_t verdict = kDraft && !finite ? kVerdictStream : kVerdictDone;
+    if (verdict == kVerdictDone) tell(verdict, 0u);
+    if (finite)
+        for (int i = tid; i < n; i += kThreads) ps.mass[i] = mass_of_key(ps.pool[i].key, a.c, M);     // read by the same thread only
+    // the keys lie between the bound and the largest, so they share the bits in which these two agree
+    const int high = 32 - __clz(top ^ sh.bound_key);
+    const uint32_t shared_bits = high < 32 ? top >> high << high : 0u;
+    const int low = DT == kBF16 ? min(16, high) : 0;       // the low 16 bits of a bf16 logit carry nothing: zeros, or
+                                                           // ones in the key of a negative one
+    const auto whole = [&](uint32_t key) { return DT == kBF16 && !(key & 0x80000000u) ? key | 0xffffu : key; };
+    const auto key_of = [&](int i) { return ps.pool[i].key; };
+    const auto mass_of = [&](int i) { return ps.mass[i]; };
+    const auto total = [&](unsigned long long v) {
+        unsigned long long t = 0;
+        block_prefix_u64(sh, v, tid, t);
+        return t;
+    };
+    const auto mass_from = [&](uint32_t key) {
         unsigned long long z = 0;
         for (int i = tid; i < n; i += kThreads)
-            if (ps.pool[i].key >= key) z += mass_of_key(ps.pool[i].key, a.c, M);
-        return block_sum_u64(sh, z, tid);
+            if (ps.pool[i].key >= key) z += ps.mass[i];
+        return total(z);
     };
+    uint32_t key_t = kTopK ? whole(pool_select<false>(sh, n, shared_bits, high, low, static_cast<uint32_t>(a.top_k), 0ull, tid,
+                                                      key_of, mass_of)) : 0u;
+    key_out = key_t;
+    if (verdict == kVerdictStream) tell(verdict, key_t);
     if (use_p && finite) {
         const unsigned long long zk = kTopK ? mass_from(key_t) : row_mass;
         if (zk > 0) {
             const unsigned long long all = kTopK ? zk : mass_from(0u);
             unsigned long long want = nucleus_target(a.top_p, zk);
             if (want > all) want = all;                // rounding at the very end of the candidates: all of them
-            key_t = max(key_t, pool_select<kLevels, true>(sh, ps.pool, n, 0u, want, a.c, M, tid));
+            key_t = max(key_t, whole(pool_select<true>(sh, n, shared_bits, high, low, 0u, want, tid, key_of, mass_of)));
         }
     }
     if (tid == 0) a.thr[row] = key_t ? key_value(key_t) : neg_inf();
-    key_out = key_t;
-    if (kDraft) {
-        tell(kVerdictStream, key_t);
-        return kVerdictStream;
+    if (verdict == kVerdictStream || (!kDraft && !a.stats)) return verdict;
+    const unsigned long long zt = finite ? mass_from(key_t) : 0ull;
+    if (tid == 0 && a.stats) a.stats[row] = kept_stats(row_max, zt, finite);
+    if (!kDraft) return verdict;
+    long long term = 0;
+    for (int i = tid; i < n; i += kThreads) {
+        if (ps.pool[i].key < key_t) { ps.mass[i] = 0; continue; }
+        const float arg = fmaxf(__fmaf_rn(key_value(ps.pool[i].key), a.c, -M), kArgFloor);
+        term += __float2ll_rz(ex2_approx(arg) * arg * kMassScale);
     }
-    tell(kVerdictDone, key_t);
-    if (a.stats) {
-        const unsigned long long zt = mass_from(key_t);
-        if (tid == 0) a.stats[row] = kept_stats(row_max, zt, finite);
+    const long long aq = static_cast<long long>(total(static_cast<unsigned long long>(term)));
+    // the sample: the first index at which the running mass of the kept candidates exceeds u * zt
+    const unsigned long long target = static_cast<unsigned long long>(static_cast<double>(a.uniforms[row]) * static_cast<double>(zt));
+    const int idx_bits = 32 - __clz(a.V);
+    const auto from_end = [&](int i) { return ~ps.pool[i].idx; };      // the lowest index has the largest key
+    const uint32_t found = ~pool_select<true>(sh, n, ~0u << idx_bits, idx_bits, 0, 0u, target + 1, tid, from_end, mass_of);
+    if (tid == 0) {
+        a.token[row] = static_cast<int32_t>(found);
+        const float Z = static_cast<float>(static_cast<double>(zt) / 1099511627776.0);
+        const float A = static_cast<float>(static_cast<double>(aq) / 1099511627776.0);
+        const float H = fmaxf(kLn2 * (log2f(Z) - A / Z), 0.f);
+        a.entropy[row] = H;
+        a.stop[row] = __fsqrt_rn(H) > a.thresh ? 1 : 0;
     }
-    return kVerdictDone;
+    return verdict;
 }
 
 // Sum of the 2^-40 fixed-point masses of elements of a row (those of mass_of_key).  Bound by instructions: nearly all elements
@@ -1073,8 +1138,9 @@ __global__ void __launch_bounds__(kThreads, 2) row_threshold_kernel(ThresholdArg
                 }
             }
         });
-        kept = block_sum_u64(sh, kept, tid);
-        if (tid == 0) sh.blk_above = kept;
+        unsigned long long of_block = 0;
+        block_prefix_u64(sh, kept, tid, of_block);
+        if (tid == 0) sh.blk_above = of_block;
         cluster.sync();
         unsigned long long all = 0;
         for (int r = 0; r < S; ++r) all += cluster.map_shared_rank(&sh, r)->blk_above;
