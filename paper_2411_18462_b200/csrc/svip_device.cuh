@@ -411,6 +411,12 @@ __device__ __forceinline__ void push4(uint32_t remote_addr, uint32_t remote_bar,
     asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
                  ::"r"(remote_addr), "r"(a), "r"(remote_bar) : "memory");
 }
+// 8 bytes of a peer's shared memory.  The peer must have released them to this block, and must not leave before it has read.
+__device__ __forceinline__ uint2 ld_remote8(uint32_t remote_addr) {
+    uint2 v;
+    asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(remote_addr) : "memory");
+    return v;
+}
 // Arrival on an mbarrier of another block of the cluster that also announces `bytes` of pushes to it.
 __device__ __forceinline__ void mbar_arrive_expect_tx_remote(uint32_t remote_bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.release.cluster.shared::cluster.b64 _, [%0], %1;"

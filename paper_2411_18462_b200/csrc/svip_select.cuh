@@ -26,7 +26,7 @@ constexpr int kHistCopies = 8;           // interleaved copies of the histogram:
                                          // lanes that meet in one bin mostly hit different words and banks
 constexpr float kMassScale = 1099511627776.0f;   // 2^40
 constexpr int kPoolCap = 2048;           // candidates of the whole cluster
-constexpr int kCandPerBlock = 1024;      // candidates one block may collect (less when blocks share the pool)
+constexpr int kCandPerBlock = 1024;      // candidates one of several blocks may collect
 constexpr int kCounted = 256;            // up to this many group maxima or candidates are put in order by counting
 constexpr int kMaxGroups = 2048;         // groups of threads whose maxima give the bound of a top-k
 
@@ -107,7 +107,8 @@ enum : uint32_t {
 struct SelectShared {
     union {
         uint32_t priv[3][256][kHistCopies];   // count, mass low word, mass high word; per digit, per copy
-        Candidate landing[kPoolCap];          // candidate path, block 0: the peers' candidates, one region per block
+        Candidate landing[kPoolCap];          // candidate path, block 0: the peers' candidates, one region per block (the
+                                              // candidates of a block alone)
     };
     union {
         alignas(16) float group_max[kMaxGroups];   // candidate path: group maxima of the whole cluster
@@ -733,18 +734,26 @@ struct MassSum {
     }
 };
 
-// Collects the elements >= t0v of the block's segments into sh.cand and (kMass) leaves the mass of all elements of every
+// Where a block collects its candidates, and lists the vectors that hold them.
+struct CollectInto {
+    Candidate* cand;
+    uint32_t cap;
+    uint32_t* vec_list;
+    uint32_t vec_cap;
+};
+
+// Collects the elements >= t0v of the block's segments and (kMass) leaves the mass of all elements of every
 // warp's segment in sh.warp_above.  `resident`: every segment of the row fits the ring and lies there since pass 1 (a
 // property of the row, so the same in every warp: a block barrier depends on it).
 template <int DT, bool kMass>
 __device__ __forceinline__ void collect(const RowGeom& g, const LaneSpan& s, bool resident, uint32_t slot0, float t0v,
-                                        uint32_t cap, SelectShared& sh, float c, float row_max) {
+                                        const CollectInto& to, SelectShared& sh, float c, float row_max) {
     constexpr int EPV = ElemTraits<DT>::kEPV;
     MassSum<DT> mass(c, row_max);
     const bool lowest = !(t0v > neg_inf());      // no bound: every element, -inf and NaN (which counts as -inf) among them
     auto take = [&](float x, int i) {
         const uint32_t pos = atomicAdd(&sh.n_cand, 1u);
-        if (pos < cap) sh.cand[pos] = Candidate{order_key(x), static_cast<uint32_t>(i)};
+        if (pos < to.cap) to.cand[pos] = Candidate{order_key(x), static_cast<uint32_t>(i)};
     };
     auto has = [&](const uint4& raw) {        // asked once per vector: it also counts its mass
         RawMax<DT> m;
@@ -778,19 +787,19 @@ __device__ __forceinline__ void collect(const RowGeom& g, const LaneSpan& s, boo
         // the streaming loop only lists the vectors, which are few, and all threads look at them afterwards: with the
         // elements looked at inside the unrolled loop, 2304 rows of 304 KB took 272 us instead of 174.  A set that
         // does not fit is of no use, so the pass ends as soon as that is known.
-        auto full = [&]() { return *static_cast<volatile uint32_t*>(&sh.n_vec) > kCandPerBlock; };
+        auto full = [&]() { return *static_cast<volatile uint32_t*>(&sh.n_vec) > to.vec_cap; };
         stream_interior(s, slot0, [&](const uint4& raw, int vi) {
             if (has(raw)) {
                 const uint32_t pos = atomicAdd(&sh.n_vec, 1u);
-                if (pos < kCandPerBlock) sh.vec_list[pos] = static_cast<uint32_t>(vi);
+                if (pos < to.vec_cap) to.vec_list[pos] = static_cast<uint32_t>(vi);
             }
         }, full);
         __syncthreads();
         const uint32_t nv = sh.n_vec;
-        if (nv > kCandPerBlock) {
-            if (threadIdx.x == 0) atomicAdd(&sh.n_cand, cap + 1);
+        if (nv > to.vec_cap) {
+            if (threadIdx.x == 0) atomicAdd(&sh.n_cand, to.cap + 1);
         } else {
-            for (uint32_t i = threadIdx.x; i < nv; i += kThreads) visit(ld_vec(g.base + sh.vec_list[i]), sh.vec_list[i]);
+            for (uint32_t i = threadIdx.x; i < nv; i += kThreads) visit(ld_vec(g.base + to.vec_list[i]), to.vec_list[i]);
         }
     }
     if (s.head) edge(0);
@@ -837,7 +846,12 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
     constexpr int EPV = ElemTraits<DT>::kEPV;
     const int lane = tid & 31, warp = tid >> 5;
     const int seg = rank * kWarps + warp;
-    const uint32_t cap = static_cast<uint32_t>(S == 1 ? kCandPerBlock : min(kCandPerBlock, kPoolCap / S));
+    // A block alone collects where the peers' candidates would land.  Otherwise every block collects at home; its first
+    // kPoolCap / S candidates are pushed to block 0, which has that much room for each, and fetches the others of a block in
+    // whose part of the row the likely tokens are gathered.
+    const CollectInto to = S == 1 ? CollectInto{sh.landing, kPoolCap, reinterpret_cast<uint32_t*>(sh.cand), 2 * kCandPerBlock}
+                                  : CollectInto{sh.cand, kCandPerBlock, sh.vec_list, kCandPerBlock};
+    const uint32_t region = kPoolCap / S;
     const int gs = group_shift(S, a.top_k);
     const int n_groups = (kWarps * S) << gs;
     uint32_t parity = 0;
@@ -899,7 +913,7 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
         const float t0v = key_value(sh.bound_key);
         pdl_launch_dependents();
         const bool resident = den == 1 && g.vps <= 32 * kStages;
-        collect<DT, !kTopK>(g, span, resident, slot0, t0v, cap, sh, a.c, row_max);
+        collect<DT, !kTopK>(g, span, resident, slot0, t0v, to, sh, a.c, row_max);
         __syncthreads();
         uint32_t verdict;
         const uint32_t mine = sh.n_cand;
@@ -909,10 +923,10 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
             for (int w = 0; w < kWarps; ++w) my_mass += sh.warp_above[w];
         }
         if (S > 1 && rank != 0) {
-            const uint32_t sent = mine <= cap ? mine : 0u;
+            const uint32_t sent = mine <= to.cap ? min(mine, region) : 0u;
             const uint32_t bar0 = map_to_rank(smem_addr(&sh.bar_pool), 0);
             for (uint32_t i = tid; i < sent; i += kThreads)
-                push8(map_to_rank(smem_addr(&sh.landing[rank * cap + i]), 0), bar0, sh.cand[i].key, sh.cand[i].idx);
+                push8(map_to_rank(smem_addr(&sh.landing[rank * region + i]), 0), bar0, sh.cand[i].key, sh.cand[i].idx);
             if (tid == 0) {
                 push16(map_to_rank(smem_addr(&sh.header[rank]), 0), bar0, mine, static_cast<uint32_t>(my_mass),
                        static_cast<uint32_t>(my_mass >> 32), 0u);
@@ -936,7 +950,6 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
             const uint32_t count = lane == 0 ? mine : head.x;
             unsigned long long row_mass = 0;
             if (!kTopK) row_mass = shfl_u64(warp_scan_mass((static_cast<unsigned long long>(head.z) << 32) | head.y, lane), 31) + my_mass;
-            const bool fits = !__any_sync(0xffffffffu, count > cap);
             uint32_t end = count;
 #pragma unroll
             for (int o = 1; o < kMaxCluster; o <<= 1) {
@@ -944,15 +957,22 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
                 if (lane >= o) end += up;
             }
             const uint32_t total = __shfl_sync(0xffffffffu, end, kMaxCluster - 1);
+            const bool fits = !__any_sync(0xffffffffu, count > to.cap) && total <= kPoolCap;
             if (!fits || total < static_cast<uint32_t>(kTopK ? a.top_k : 1)) {
                 verdict = !fits && den > 1 ? kVerdictRetry : kVerdictDescend;
                 tell(verdict, 0u);
             } else {
                 // two warps copy the candidates of each block
                 const int r = warp & (kMaxCluster - 1);
-                const uint32_t nr = __shfl_sync(0xffffffffu, count, r), to = __shfl_sync(0xffffffffu, end, r) - nr;
-                const Candidate* from = r == 0 ? sh.cand : sh.landing + r * cap;
-                for (uint32_t t = (warp / kMaxCluster) * 32 + lane; t < nr; t += 64) scratch->pool[to + t] = from[t];
+                const uint32_t nr = __shfl_sync(0xffffffffu, count, r), first = __shfl_sync(0xffffffffu, end, r) - nr;
+                const uint32_t here = r == 0 ? nr : min(nr, region);
+                const Candidate* from = r == 0 ? to.cand : sh.landing + r * region;
+                for (uint32_t t = (warp / kMaxCluster) * 32 + lane; t < here; t += 64) scratch->pool[first + t] = from[t];
+                // the block stays, and keeps its candidates, until it hears the verdict
+                for (uint32_t t = here + (warp / kMaxCluster) * 32 + lane; t < nr; t += 64) {
+                    const uint2 o = ld_remote8(map_to_rank(smem_addr(&sh.cand[t]), r));
+                    scratch->pool[first + t] = Candidate{o.x, o.y};
+                }
                 __syncthreads();
                 verdict = finish_pool<DT, kDraft, kTopK>(sh, *scratch, static_cast<int>(total), a, use_p, row_mass, row, tid,
                                                   key_out, tell);
