@@ -193,7 +193,9 @@ int pick_draft_cluster(const svip_ctx* ctx, long rows, int V, int dtype) {
 //            or 8 blocks, 9.7 with 3, 10.6 with 6); 6 where with 4 the segments do not fit the ring (32 rows of 304 KB:
 //            12.7 us with 6, 14.0 with 4; 36 of 1 MB 16.9 and 21.1)
 //   nucleus  6, 4, 3 for long rows, 2 (16 rows of 304 KB: 10.6 us with 6, 11.5 with 8; 72 rows: 14.8 with 3, 16.2 with 2,
-//            but 9.8 and 9.5 for rows of 128 KB)
+//            but 9.8 and 9.5 for rows of 128 KB); 8 up to 8 rows, where it costs little and flat rows, which take the descent,
+//            gain more (8 rows of 608 KB 11.2 us with 8, 10.8 with 6, flat 42.8 and 48.1; of 512 KB 11.1 and 11.7, flat 37.1
+//            and 43.2; of 1 MB 13.8 and 12.5, flat 54.6 and 62.4; 16 rows of 608 KB 13.9 and 12.1, flat 57.4 and 55.2)
 // and 2 rather than 1 as long as it fits (144 rows of 304 KB: 18.0 against 21.4 us).  Launches that fit with no size
 // are cut as those of the other kernels.
 int pick_threshold_cluster(const svip_ctx* ctx, long rows, int V, int dtype, bool top_k) {
@@ -203,7 +205,7 @@ int pick_threshold_cluster(const svip_ctx* ctx, long rows, int V, int dtype, boo
     const int sizes[] = {8, 6, 4, 3, 2};
     for (const int S : sizes) {
         if (rows > ctx->max_clusters[S] - 2 || nvec < static_cast<long>(S) * kThreads) continue;
-        if (top_k ? S == 3 || (S == 6 && resident(4)) : S == 8 || (S == 3 && nvec * 16 < (256L << 10))) continue;
+        if (top_k ? S == 3 || (S == 6 && resident(4)) : (S == 8 && rows > 8) || (S == 3 && nvec * 16 < (256L << 10))) continue;
         return S;
     }
     return pick_cluster(ctx, rows, V, dtype);

@@ -658,10 +658,11 @@ __device__ __forceinline__ void stream_interior(const LaneSpan& s, uint32_t slot
     for (; it < s.n; ++it) f(lds128(slot0 + (it & (kStages - 1)) * kSlotStride), s.vi0 + 32 * it);
 }
 
-// The same over vectors that are still in the ring, after a pass over a span of at most kStages vectors per lane.
-template <class F>
-__device__ __forceinline__ void revisit_interior(const LaneSpan& s, uint32_t slot0, F&& f) {
-    for (int it = 0; it < s.n; ++it) f(lds128(slot0 + it * (kThreads * 16)), s.vi0 + 32 * it);
+// The same over vectors that are still in the ring, after a pass over a span of at most kStages vectors per lane.  stop() is
+// asked before every vector.
+template <class F, class Stop = NeverStop>
+__device__ __forceinline__ void revisit_interior(const LaneSpan& s, uint32_t slot0, F&& f, Stop&& stop = Stop()) {
+    for (int it = 0; it < s.n && !stop(); ++it) f(lds128(slot0 + it * (kThreads * 16)), s.vi0 + 32 * it);
 }
 
 // Streams segment `seg` of the row with the calling warp and returns the warp's merged partial

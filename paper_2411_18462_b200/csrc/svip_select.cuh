@@ -751,10 +751,13 @@ __device__ __forceinline__ void collect(const RowGeom& g, const LaneSpan& s, boo
     constexpr int EPV = ElemTraits<DT>::kEPV;
     MassSum<DT> mass(c, row_max);
     const bool lowest = !(t0v > neg_inf());      // no bound: every element, -inf and NaN (which counts as -inf) among them
-    auto take = [&](float x, int i) {
-        const uint32_t pos = atomicAdd(&sh.n_cand, 1u);
+    auto place = [&](float x, uint32_t pos, int i) {
         if (pos < to.cap) to.cand[pos] = Candidate{order_key(x), static_cast<uint32_t>(i)};
     };
+    // A set that does not fit is of no use, and a flat row has tens of thousands of elements above the bound, each of which
+    // would wait for its turn at the counter: collecting ends as soon as that is known, and a vector asks for all its places
+    // at once (draft step with Gaussian logits, top-p 0.9: 1 row of 304 KB 39.3 -> 31.7 us, 384 rows of 64 KB 90 -> 74).
+    auto over = [&]() { return *static_cast<volatile uint32_t*>(&sh.n_cand) > to.cap; };
     auto has = [&](const uint4& raw) {        // asked once per vector: it also counts its mass
         RawMax<DT> m;
         m.reset();
@@ -766,9 +769,14 @@ __device__ __forceinline__ void collect(const RowGeom& g, const LaneSpan& s, boo
     auto visit = [&](const uint4& raw, int vi) {
         float x[EPV];
         ElemTraits<DT>::unpack(raw, x);
+        uint32_t hits = 0;
+#pragma unroll
+        for (int j = 0; j < EPV; ++j) hits += x[j] >= t0v || lowest ? 1u : 0u;
+        if (hits == 0 || over()) return;
+        uint32_t pos = atomicAdd(&sh.n_cand, hits);
 #pragma unroll
         for (int j = 0; j < EPV; ++j)
-            if (x[j] >= t0v || lowest) take(x[j], vi * EPV + j - g.pre);
+            if (x[j] >= t0v || lowest) place(x[j], pos++, vi * EPV + j - g.pre);
     };
     auto edge = [&](int vi) {
         float x[EPV];
@@ -778,18 +786,19 @@ __device__ __forceinline__ void collect(const RowGeom& g, const LaneSpan& s, boo
             const int i = vi * EPV + j - g.pre;
             if (i < 0 || i >= g.V) continue;
             if (kMass) mass.one(x[j]);
-            if (x[j] >= t0v || lowest) take(x[j], i);
+            if (x[j] >= t0v || lowest) place(x[j], atomicAdd(&sh.n_cand, 1u), i);
         }
     };
     if (resident) {
-        revisit_interior(s, slot0, [&](const uint4& raw, int vi) { if (has(raw)) visit(raw, vi); });
+        const auto look = [&](const uint4& raw, int vi) { if (has(raw)) visit(raw, vi); };
+        if constexpr (kMass) revisit_interior(s, slot0, look, over);
+        else revisit_interior(s, slot0, look);
     } else {
         // the streaming loop only lists the vectors, which are few, and all threads look at them afterwards: with the
-        // elements looked at inside the unrolled loop, 2304 rows of 304 KB took 272 us instead of 174.  A set that
-        // does not fit is of no use, so the pass ends as soon as that is known.
+        // elements looked at inside the unrolled loop, 2304 rows of 304 KB took 272 us instead of 174
         auto full = [&]() { return *static_cast<volatile uint32_t*>(&sh.n_vec) > to.vec_cap; };
         stream_interior(s, slot0, [&](const uint4& raw, int vi) {
-            if (has(raw)) {
+            if (has(raw) && !full()) {
                 const uint32_t pos = atomicAdd(&sh.n_vec, 1u);
                 if (pos < to.vec_cap) to.vec_list[pos] = static_cast<uint32_t>(vi);
             }

@@ -138,3 +138,13 @@ def test_gathered_sets_cost_what_spread_ones_do(ctx):
     for B, V, n in ((16, 152064, 700), (1, 152064, 400)):
         spread = us_per_call(ctx, W.to_bf16_bits(planted(rng, B, V, n)), 0, 0.9)
         assert us_per_call(ctx, W.to_bf16_bits(planted(rng, B, V, n, 0.0, 0.1)), 0, 0.9) < 1.35 * spread, (B, V, n)
+
+
+def test_flat_rows_leave_the_candidates_soon(ctx):
+    # a nucleus of tens of thousands of tokens takes the descent by mass; with a top-k that drops nothing but one token the
+    # row takes the same descent after one by counts.  Measured 0.92 of that; collecting to the end 1.1
+    rng = np.random.default_rng(4)
+    for B, V in ((300, 32000), (16, 152064)):
+        x = -1.1 * np.log(np.arange(1, V + 1))
+        rows = W.to_bf16_bits(np.stack([x[rng.permutation(V)] for _ in range(B)]).astype(np.float32))
+        assert us_per_call(ctx, rows, 0, 0.95) < 1.02 * us_per_call(ctx, rows, V - 1, 0.95), (B, V)
