@@ -23,7 +23,7 @@ namespace svip {
 // (0.97 GB moved for 0.62 GB) all at once, so instructions were taken out: packed arithmetic in phase 2, loops unrolled
 // over the ring, one small merge per block.  1024 pairs of 152064 bf16 logits 190 -> 156 us, of 256000 fp32 593 -> 476 (with the lines of the second pass given up first).
 // Segments whose fast sums are not finite (-inf / NaN logits, rows that start far below their
-// maximum, vectors that stick out of the row) are summed again by an exact masking path.
+// maximum) are summed again by an exact masking path.
 
 struct PairArgs {
     const void* t_logits;
@@ -75,7 +75,7 @@ __device__ __forceinline__ PairPartial pair_warp_merge(PairPartial t, float c) {
 }
 
 // Streams warp segment `seg` of the two rows together: vectors inside both rows go through the
-// ring (four stages per row), the ones that stick out of a row are handed over masked to -inf by
+// ring (four stages per row), the ones that stick out of a row are handed over masked by
 // lane 0; rows of different 16-byte phase are read element by element.  f(x, d) gets the target and
 // draft logits of one vector.  kBackward walks the lane's vectors from the last to the first: a second pass over
 // rows that were just streamed meets the most recently read lines first, which are the ones L2 still
@@ -89,16 +89,18 @@ __device__ __forceinline__ void stream_pair(const RowGeom& g, const RowGeom& gq,
     constexpr int kDepth = kStages / 2;
     int v_lo, v_hi;
     seg_range(g, seg, v_lo, v_hi);
+    // elements outside the rows get a finite stand-in that weighs nothing: -inf would make 0 * -inf = NaN of the sums, and
+    // the segment would be summed again element by element (the two segments at the ends of a row nearly always have some)
     auto masked = [&](int vi) {
         float x[EPV], d[EPV];
-        unpack_masked<DT>(ld_vec(g.base + vi), vi, g, x);
+        unpack_edge<DT>(ld_vec(g.base + vi), vi, g, x);
         if (gq.pre == g.pre) {
-            unpack_masked<DT>(ld_vec(gq.base + vi), vi, gq, d);
+            unpack_edge<DT>(ld_vec(gq.base + vi), vi, gq, d);
         } else {
 #pragma unroll
             for (int j = 0; j < EPV; ++j) {
                 const int i = vi * EPV + j - g.pre;
-                d[j] = (i >= 0 && i < g.V) ? ElemTraits<DT>::load_one(qrow, i) : neg_inf();
+                d[j] = (i >= 0 && i < g.V) ? ElemTraits<DT>::load_one(qrow, i) : kMasked;
             }
         }
         f(x, d);
