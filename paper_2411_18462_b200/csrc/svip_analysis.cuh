@@ -463,7 +463,18 @@ __global__ void __launch_bounds__(kThreads, 2) pair_stats_kernel(PairArgs a) {
             unpack2(b2, b0, b1);
             beta = warp_sum(b0 + b1);
         } else {
-            pair_segment_exact<DT>(gt, gq, qrow, seg, a.c, lane, kp, kq, &beta);
+            // the same for masked logits: NaN counts as -inf, whose exponential is 0
+            float b1 = 0.f;
+            stream_pair<DT, true>(gt, gq, qrow, seg, lane, slot0, [&](const float (&x)[EPV], const float (&d)[EPV]) {
+#pragma unroll
+                for (int j = 0; j < EPV; j += 2) {
+                    beta += ex2_approx(fminf(__fmaf_rn(fmaxf(x[j], neg_inf()), a.c, -kp),
+                                             __fmaf_rn(fmaxf(d[j], neg_inf()), a.c, -kq)));
+                    b1 += ex2_approx(fminf(__fmaf_rn(fmaxf(x[j + 1], neg_inf()), a.c, -kp),
+                                           __fmaf_rn(fmaxf(d[j + 1], neg_inf()), a.c, -kq)));
+                }
+            }, primed);
+            beta = warp_sum(beta + b1);
         }
     }
     if (S == 1) {
