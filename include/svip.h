@@ -109,7 +109,7 @@ int svip_set_cluster_size(svip_ctx* ctx, int cluster_size);
 /*
  * Number of kernels this context has launched (or recorded into a graph) so far.
  * A policy step that the draft kernel of a drafting loop takes over (see
- * svip_graph_loop_begin) counts as one.
+ * svip_graph_loop_begin) is no kernel and is not counted.
  */
 long svip_launch_count(const svip_ctx* ctx);
 

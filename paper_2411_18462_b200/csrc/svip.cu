@@ -928,8 +928,7 @@ int svip_policy_advance(svip_ctx* ctx, int policy, const uint8_t* stop, const in
     if (decides) a.loop = ctx->loop;
     a.arrived = nullptr;
     if (decides && join_draft_step(ctx, a)) {
-        ctx->loop_decided = 1;
-        ctx->launches += 1;      // counted like the kernel it replaces
+        ctx->loop_decided = 1;      // no kernel of its own: nothing to count
         return SVIP_OK;
     }
     cudaError_t e = launch_ex(policy_advance_kernel, 1, kPolicyThreads, 0, 0, static_cast<cudaStream_t>(stream), a);

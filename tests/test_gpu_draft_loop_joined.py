@@ -37,6 +37,7 @@ def test_joined_and_separate_policy_step_agree(ctx, B, V, T, policy, max_iters):
         bufs["act"][B // 2:B // 2 + 1] = 1 if B == 1 else 0        # one sequence is not drafting
         torch.cuda.synchronize()
         st = torch.cuda.Stream()
+        before = ctx.launch_count()
         ctx.graph_begin(st)
         body = ctx.graph_loop_begin(st, bufs["nact"], max_iters)
         ctx.draft_step_at(bufs["q"], tl.dtype_code(w.q_logits), B, V, V, B * V, bufs["len"], B, T, w.h, bufs["ud"], bufs["act"],
@@ -46,6 +47,7 @@ def test_joined_and_separate_policy_step_agree(ctx, B, V, T, policy, max_iters):
         ctx.policy_advance(policy, bufs["stop"], bufs["gamma"], bufs["len"], bufs["act"], B, K_cap, bufs["nact"], stream=body)
         ctx.graph_loop_end()
         graph = ctx.graph_end(st)
+        assert ctx.launch_count() - before == (3 if apart else 1)    # draft step, packing, policy step, or the draft step alone
         seen = []
         for replay in range(2):                                      # the second one starts where the first one ended
             graph.launch(st)
