@@ -14,7 +14,9 @@ travels with the source tree; it is never installed into site-packages.
 """
 from __future__ import annotations
 
+import hashlib
 import os
+import re
 import shutil
 import subprocess
 import sys
@@ -35,21 +37,37 @@ NATIVE_SOURCE = os.path.join(CSRC, "native_calls.cpp")
 NATIVE = os.path.join(CSRC, "native_calls" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 
+def abi_fingerprint() -> str:
+    """Identifies the C ABI: what include/svip.h says apart from its comments."""
+    with open(os.path.join(INCLUDE, "svip.h")) as f:
+        text = re.sub(r"/\*.*?\*/", " ", f.read(), flags=re.S)
+    return hashlib.sha256(" ".join(text.split()).encode()).hexdigest()[:16]
+
+
 def build_native(force: bool = False):
     """The argument-converting extension; None where it cannot be built (binding.py then uses ctypes)."""
     python_h = sysconfig.get_paths()["include"]
     deps = [NATIVE_SOURCE, os.path.join(INCLUDE, "svip.h")]
     if not force and os.path.exists(NATIVE) and all(os.path.getmtime(d) <= os.path.getmtime(NATIVE) for d in deps):
         return NATIVE
+    why = None
     cxx = shutil.which("g++")
-    if not cxx or not os.path.exists(os.path.join(python_h, "Python.h")):
-        print("native_calls: no g++ or no Python.h, the binding uses ctypes", file=sys.stderr)
-        return None
     tmp = NATIVE + ".%d.tmp" % os.getpid()
-    subprocess.check_call([cxx, "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-I", python_h, "-I", INCLUDE,
-                           "-o", tmp, NATIVE_SOURCE])
-    os.replace(tmp, NATIVE)
-    return NATIVE
+    if not cxx or not os.path.exists(os.path.join(python_h, "Python.h")):
+        why = "no g++ or no Python.h"
+    else:
+        try:
+            subprocess.check_call([cxx, "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-I", python_h, "-I", INCLUDE,
+                                   '-DSVIP_ABI_FINGERPRINT="%s"' % abi_fingerprint(), "-o", tmp, NATIVE_SOURCE])
+            os.replace(tmp, NATIVE)
+            return NATIVE
+        except (subprocess.CalledProcessError, OSError) as e:
+            why = str(e)
+    for stale in (tmp, NATIVE):        # one of other sources must not be loaded in its place
+        if os.path.exists(stale):
+            os.remove(stale)
+    print("native_calls: %s, the binding uses ctypes" % why, file=sys.stderr)
+    return None
 
 
 def _nvcc() -> str:
