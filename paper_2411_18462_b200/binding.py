@@ -151,6 +151,12 @@ def _load_calls(L):
     loader = importlib.machinery.ExtensionFileLoader("native_calls", path)
     native = importlib.util.module_from_spec(importlib.util.spec_from_file_location("native_calls", path, loader=loader))
     loader.exec_module(native)
+    # an extension of another header would call the library with shifted arguments (without the header beside the package
+    # there is nothing to compare, and nothing that could have changed)
+    from . import build
+    if os.path.exists(os.path.join(build.INCLUDE, "svip.h")) and \
+            getattr(native, "abi_fingerprint", "") != build.abi_fingerprint():
+        return _CtypesCalls(L)
     native.load({n: C.cast(getattr(L, "svip_" + n), C.c_void_p).value for n in _CALL_NAMES})
     return native
 

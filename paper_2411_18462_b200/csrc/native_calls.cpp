@@ -137,9 +137,16 @@ PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "native_calls", nullptr, -1, g_me
 
 }  // namespace
 
+#ifndef SVIP_ABI_FINGERPRINT
+#define SVIP_ABI_FINGERPRINT ""
+#endif
+
 PyMODINIT_FUNC PyInit_native_calls(void) {
     g_data_ptr = PyUnicode_InternFromString("data_ptr");
     g_cuda_stream = PyUnicode_InternFromString("cuda_stream");
     if (!g_data_ptr || !g_cuda_stream) return nullptr;
-    return PyModule_Create(&g_module);
+    PyObject* m = PyModule_Create(&g_module);
+    // the function types above are those of the header this was compiled with; binding.py compares
+    if (m && PyModule_AddStringConstant(m, "abi_fingerprint", SVIP_ABI_FINGERPRINT) < 0) { Py_DECREF(m); return nullptr; }
+    return m;
 }
