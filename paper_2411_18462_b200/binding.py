@@ -406,7 +406,8 @@ class Context:
         argtypes = entry.argtypes
         if len(args) != len(argtypes) - 1:
             raise TypeError("svip_%s takes %d arguments after the context, %d given" % (name, len(argtypes) - 1, len(args)))
-        conv = tuple(_convert(a, t) for a, t in zip(args, argtypes[1:]))
+        # through the ctypes types, which take no fraction for an integer and no text for a number
+        conv = tuple(t(_convert(a, t) if t is C.c_void_p else a).value for a, t in zip(args, argtypes[1:]))
         fn, h, hv = getattr(_calls, name, entry), self._h, self._hv
 
         def call():

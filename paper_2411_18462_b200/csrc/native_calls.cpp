@@ -49,9 +49,11 @@ template <class T> struct Arg<T*> {
 };
 template <> struct Arg<float> {
     static bool get(PyObject* o, bool, float* out) {
-        const double d = PyFloat_AsDouble(o);
-        if (d == -1.0 && PyErr_Occurred()) return false;
-        *out = static_cast<float>(d);
+        if (PyFloat_CheckExact(o)) { *out = static_cast<float>(PyFloat_AS_DOUBLE(o)); return true; }
+        PyObject* v = PyNumber_Float(o);      // what float() takes, texts included
+        if (!v) return false;
+        *out = static_cast<float>(PyFloat_AS_DOUBLE(v));
+        Py_DECREF(v);
         return true;
     }
 };

@@ -54,3 +54,18 @@ def test_bad_arguments_raise(calls):
             draft(c.draft_step, 0, logits=object())
         with pytest.raises((TypeError, ValueError)):
             draft(c.draft_step, 0, T="warm")
+
+
+def test_what_the_conversions_take_and_refuse(calls):
+    from paper_2411_18462_b200 import binding
+    for c in calls:
+        assert draft(c.draft_step, C.addressof(C.create_string_buffer(4096)), T="1.0", B=0.0) == 0    # as float() and int() do
+    ctx = object.__new__(binding.Context)
+    ctx._h, ctx._hv = C.c_void_p(), 0
+    args = dict(logits=Tensor(), dtype=0, B=0, V=8, stride=8, T=1.0, thresh=0.3, uniforms=Tensor(), token=1 << 20, entropy=Tensor(),
+                stop=Tensor(), stats=None, stream=Stream())
+    with pytest.raises(binding.SvipError):
+        ctx.bind("draft_step", *args.values())()           # no context: the library refuses it
+    for over in (dict(B=2.5), dict(V="8"), dict(T="1.0"), dict(dtype=None)):
+        with pytest.raises(TypeError):
+            ctx.bind("draft_step", *dict(args, **over).values())
