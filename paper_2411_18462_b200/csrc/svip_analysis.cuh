@@ -66,14 +66,6 @@ __device__ __forceinline__ void pair_rescale(PairPartial& t, float Mp, float Mq,
     t.mp = Mp; t.mq = Mq;
 }
 
-// All lanes return the merge of the 32 lanes' partials.
-__device__ __forceinline__ PairPartial pair_warp_merge(PairPartial t, float c) {
-    const float Mp = warp_max(t.mp), Mq = warp_max(t.mq);
-    pair_rescale(t, Mp, Mq, c);
-    t.Zp = warp_sum(t.Zp); t.Zq = warp_sum(t.Zq); t.Aq = warp_sum(t.Aq); t.D = warp_sum(t.D);
-    return t;
-}
-
 // Streams warp segment `seg` of the two rows together: vectors inside both rows go through the
 // ring (four stages per row), the ones that stick out of a row are handed over masked by
 // lane 0; rows of different 16-byte phase are read element by element.  f(x, d) gets the target and

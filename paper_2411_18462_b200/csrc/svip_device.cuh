@@ -836,33 +836,14 @@ __device__ __forceinline__ float warp_scan_incl(float v, int lane) {
     return v;
 }
 
-// Block-wide exclusive scan of one float per thread; also returns the block total.
-// `wsum` is shared scratch of kWarps floats.  Contains two __syncthreads().
-__device__ __forceinline__ float block_scan_excl(float v, float* wsum, int lane, int warp, float& total) {
-    float inc = warp_scan_incl(v, lane);
-    __syncthreads();   // wsum may still be read from the previous round
-    if (lane == 31) wsum[warp] = inc;
-    __syncthreads();
-    float before = 0.f, tot = 0.f;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) {
-        float s = wsum[w];
-        if (w < warp) before += s;
-        tot += s;
-    }
-    total = tot;
-    return before + (inc - v);
-}
-
 // ---------------------------------------------------------------------------
 // Locating a sample among the segments of a row.
 //
-// Each block of the cluster publishes, per warp, the mass of its segment in
-// shared memory.  Warp 0 of EVERY block then reads all segments of the cluster
-// through distributed shared memory, in the same order with the same
-// arithmetic, so all blocks agree bit for bit on the total, on the target mass
-// u * total and on the segment that holds it; the block that owns the segment
-// does the fine scan.
+// Every warp pushes the mass of its segment into the shared memory of every block
+// of the cluster.  Warp 0 of EVERY block then reads all segments from its own
+// block's table, in the same order with the same arithmetic, so all blocks agree
+// bit for bit on the total, on the target mass u * total and on the segment that
+// holds it; the block that owns the segment does the fine scan.
 
 struct SegPick {
     float total;    // sum of all segment masses = last inclusive prefix

@@ -87,12 +87,17 @@ def test_bound_from_half_of_the_row_lets_too_many_in(ctx, oracle):
     rng = np.random.default_rng(5)
     x = rng.standard_normal((n, V)).astype(np.float32)
     x[::7] -= 20.0
-    for S, rows in ((1, x), (2, x)):
+    for S in (1, 2):
+        rows = x.copy()
         nseg = 16 * S
         vps = ((V // 4 + nseg - 1) // nseg + 7) // 8 * 8
+        first = np.zeros(V, dtype=bool)
         for seg in range(nseg):
             lo = seg * vps * 4
+            first[lo:min(lo + vps * 2, V)] = True
             rows[::7, lo + vps * 2:min(lo + vps * 4, V)] += 20.0 / 2
+        for row in rows[::7]:      # what the first half bounds from below does not fit the tables (2048), so there is a second bound
+            assert (row >= np.sort(row[first])[-50]).sum() > 2048
         ctx.set_cluster_size(S)
         try:
             for k, p in ((50, 1.0), (50, 0.9)):
