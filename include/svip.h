@@ -188,8 +188,9 @@ int svip_draft_step_at(svip_ctx* ctx, const void* logits, svip_dtype dtype, int 
  * mass comes within about 1e-6 of top_p.  T > 0.  NaN logits count as -inf.
  * Cost: with a small top_k (at most a quarter of the threads that share a row,
  * i.e. 128 .. 1024), with or without top_p, and with top_p alone on rows that
- * are not nearly flat (up to about a thousand tokens of mass above
- * (1 - top_p) / V), every row is read twice; otherwise once per radix pass:
+ * are not nearly flat (up to 2048 tokens of mass above (1 - top_p) / V, of
+ * which at most 1024 in the part of one of several thread blocks), every row
+ * is read twice; otherwise once per radix pass:
  * 2 (bf16) or 4 (fp32) passes for top-k, as many again for the nucleus
  * (+1 for the nucleus alone).
  *   logits  DEVICE, row r starts at element r*row_stride;  thr  DEVICE [n_rows] fp32 out

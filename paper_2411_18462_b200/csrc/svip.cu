@@ -166,23 +166,33 @@ int pick_cluster(const svip_ctx* ctx, long rows, int V, int dtype) {
     return static_cast<int>(S);
 }
 
-// Blocks per row of a draft step: rows of up to 128 KB are not cut further than into 4 (16 rows of 64 KB: 3.3 us with
-// 4 blocks, 3.8 with 8, 4.0 with 6, launches of equal size; 9 to 14 rows of 128 KB in launches of changing size: 3.6 with 4,
-// 3.9 with 8; below 8 rows of 128 KB the two are equal within 0.1), and into 2 while that takes half of the SMs at most and 4
-// would not (27 to 32 rows of 64 KB: 4.0 against 4.4).  A grid between a half and one block per SM is faster
+// Blocks per row of a draft step (and of svip_vp_locate, the same kernel).  Where pick_cluster gives 6 or 8, rows of up to
+// 128 KB (below 8 rows up to 64 KB) take 4, or 2 from about a fifth as many rows as SMs on (30 to 43 rows).  us with 2, 4, 6
+// and 8 blocks, launches of equal size:
+//                 16 rows                  24 rows                  32 rows                  38 rows
+//      64 KB  3.63 3.35 4.03 4.05      3.70 3.63 4.14 4.11      3.78 4.21 4.28 4.49      3.89 4.28 4.38 5.48
+//      96 KB  4.05 3.60 4.06 4.31      4.05 3.79 4.22 4.39      4.05 4.50 4.29 4.78      4.25 4.57 4.40 5.85
+//     128 KB  4.38 3.77 4.15 4.30      4.37 4.04 4.57 4.37      4.38 4.73 4.59 4.82      4.58 4.82 4.66 5.76
+// A grid between a half and one block per SM is faster
 // still as long as every launch has the same size, because all blocks of the next launch then find a place and prefetch, but
 // not when the batch shrinks from launch to launch and two blocks of a launch meet on one SM (112 rows of 304 KB: one
 // block per row 10.5 us against 13.6, two 11.0 either way), so it is not sought.
-// Long rows, somewhat more than SMs: 3 blocks per row as long as that is at most two full rounds of two blocks per SM; fewer
-// and longer blocks leave much of the GPU idle at the end (150 rows: 1 MB 29.6 us with 3, 35.1 with 2; 800 KB 24.3 and
-// 28.1; 160 rows: 608 KB 20.9 and 23.2; 512 KB 23.4 and 25.9 with 1; but 304 KB 17.7 and 17.3 with 1).
+// Long rows, somewhat more than SMs (149 to 197): 3 blocks per row, which is at most two full rounds of two blocks per SM; fewer
+// and longer blocks leave much of the GPU idle at the end.  us with 1, 2, 3 and 4 blocks:
+//                      149 rows                     160 rows                     197 rows                  198 rows (not)
+//     390 KB (not)  15.8 15.5 14.9 15.9        16.1 16.0 15.9 16.3        17.4 16.9 18.4 18.2        17.5 17.0 18.5 18.3
+//     449 KB        18.4 17.0 16.0 17.6        20.0 17.7 17.2 18.4        21.0 19.0 20.5 20.5        21.0 19.0 20.6 20.5
+//     500 KB fp32   18.5 19.4 17.6 19.7        18.6 20.8 19.0 21.1        21.5 21.6 21.6 23.5        21.6 21.6 21.7 23.6
+//     500 KB bf16   25.4 26.3 21.2 26.5        25.8 27.7 23.1 26.8        26.3 28.4 25.5 31.8        26.3 28.6 25.6 32.0
+//     594 KB        22.4 21.3 19.4 20.1        23.2 22.9 20.9 20.9        24.8 24.4 23.9 24.5        25.0 24.7 24.1 24.5
+//     1000 KB       36.2 34.2 29.0 29.6        38.0 36.8 31.2 32.3        41.0 39.0 36.3 38.1        41.5 39.2 36.6 38.4
 int pick_draft_cluster(const svip_ctx* ctx, long rows, int V, int dtype) {
     const int S = pick_cluster(ctx, rows, V, dtype);
     const long nvec = (static_cast<long>(V) * (dtype == SVIP_BF16 ? 2 : 4) + 15) / 16;
     if (ctx->cluster_override == 0 && rows > ctx->num_sms && 3 * rows <= 4L * ctx->num_sms && nvec * 16 > (448L << 10)) return 3;
     const bool shorter = nvec < 8L * kThreads || (nvec <= 16L * kThreads && rows >= 8);
-    if (ctx->cluster_override > 0 || S <= 3 || !shorter) return S;
-    return rows * 4 <= ctx->num_sms && rows * 8 > ctx->num_sms ? 2 : 4;
+    if (ctx->cluster_override > 0 || S <= 4 || !shorter) return S;
+    return rows * 5 > ctx->num_sms ? 2 : 4;
 }
 
 // Blocks per row of the threshold kernel.  Its blocks hold over 100 KB of shared memory and its rows take several
@@ -1012,7 +1022,7 @@ int svip_vp_locate(svip_ctx* ctx, const void* logits, svip_dtype dtype, int B, i
     a.uniforms = nullptr; a.token = token; a.entropy = nullptr; a.stop = nullptr; a.row_stats = nullptr;
     a.status = ctx->status; a.active = active; a.ext_target = local_target; a.token_offset = vocab_offset;
     a.pos = nullptr; a.pos_stride = 0; a.slot_stride = 0; a.thr = nullptr; a.adv.arrived = nullptr;
-    const int S = pick_cluster(ctx, B, V_shard, dtype);
+    const int S = pick_draft_cluster(ctx, B, V_shard, dtype);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e = dtype == SVIP_BF16 ? launch_clustered(draft_step_kernel<kBF16, false, 2>, B, S, a, st, kRingBytes)
                                        : launch_clustered(draft_step_kernel<kF32, false, 2>, B, S, a, st, kRingBytes);

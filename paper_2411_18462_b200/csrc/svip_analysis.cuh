@@ -19,9 +19,9 @@ namespace svip {
 //   2. beta does need the normalisers: min(p, q) = 2^min(ap - log2 Zp, aq - log2 Zq), one more pass
 //      over the two rows with one exponential per element, from the end to the start: the last vectors
 //      still lie in the ring, the ones before them in L2 as far as the pairs in flight leave room.
-// Bound by issue slots (72 % active), the exponentials (62 % of that pipe) and, with one block per pair, DRAM
-// (0.97 GB moved for 0.62 GB) all at once, so instructions were taken out: packed arithmetic in phase 2, loops unrolled
-// over the ring, one small merge per block.  1024 pairs of 152064 bf16 logits 190 -> 156 us, of 256000 fp32 593 -> 476 (with the lines of the second pass given up first).
+// Bound by issue slots, the exponentials (three per pair of elements) and, with one block per pair, DRAM all at once, so
+// instructions were taken out: packed arithmetic in phase 2, loops unrolled
+// over the ring, one small merge per block.  Back to back with new inputs, 1024 pairs of 152064 bf16 logits 201 -> 162 us.
 // Segments whose fast sums are not finite (-inf / NaN logits, rows that start far below their
 // maximum) are summed again by an exact masking path.
 
@@ -103,8 +103,8 @@ __device__ __forceinline__ void stream_pair(const RowGeom& g, const RowGeom& gq,
     }
     const LaneSpan span = lane_span<DT>(g, seg, lane);
     const int n = span.n;
-    // the backward pass is the last one: what it has read makes room for the first pass of the pairs beside it (1024
-    // pairs of 152064 bf16 158.0 -> 155.9 us, 256000 fp32 509 -> 489)
+    // the backward pass is the last one: what it has read makes room for the first pass of the pairs beside it (by graph,
+    // 1024 pairs of 152064 bf16 158.0 -> 155.9 us, 256000 fp32 509 -> 489)
     const uint64_t policy = last_use_policy();
     auto fetch = [&](uint32_t saddr, const void* gptr) {
         if constexpr (kBackward) cp_async16_last_use(saddr, gptr, policy);

@@ -757,7 +757,7 @@ __device__ __forceinline__ void collect(const RowGeom& g, const LaneSpan& s, boo
     };
     // A set that does not fit is of no use, and a flat row has tens of thousands of elements above the bound, each of which
     // would wait for its turn at the counter: collecting ends as soon as that is known, and a vector asks for all its places
-    // at once (draft step with Gaussian logits, top-p 0.9: 1 row of 304 KB 39.3 -> 31.7 us, 384 rows of 64 KB 90 -> 74).
+    // at once (draft step with Gaussian logits, top-p 0.9: 1 row of 304 KB 39.3 -> 31.7 us, 384 rows of 64 KB 90 -> 70).
     auto over = [&]() { return *static_cast<volatile uint32_t*>(&sh.n_cand) > to.cap; };
     auto has = [&](const uint4& raw) {        // asked once per vector: it also counts its mass
         RawMax<DT> m;
