@@ -37,10 +37,9 @@ FALLBACK_HBM_GBS = 6650.0
 # ncu capture of a 1056-row launch (321.20 MB read and 10.73 MB written for 321.16 MB of logits); traffic
 # grows in proportion to the rows, so a full launch is scaled by its bytes
 ROW_STATS_TRAFFIC_PER_ALGORITHMIC_BYTE = 331.93 / 321.16
-# the same for draft_step_kernel<f32, sampling> in the launch shape timed on `stress` (clusters of 2,
-# three blocks per SM), from a capture of 160-row launches (166.44 MB read and 9.27 MB written for
-# 163.84 MB of logits)
-DRAFT_F32_TRAFFIC_PER_ALGORITHMIC_BYTE = 175.71 / 163.84
+# the same for draft_step_kernel<f32, sampling> in the launch timed on `stress` (256 rows, clusters of 2, three
+# blocks per SM): 266.23 MB read and 9.06 MB written for 262.14 MB of logits
+DRAFT_F32_TRAFFIC_PER_ALGORITHMIC_BYTE = 275.29 / 262.14
 
 
 def describe(w, B=None):
