@@ -472,6 +472,7 @@ template <> struct RawMax<kF32> {
         m = max3(m, __uint_as_float(v.x), __uint_as_float(v.y));
         m = max3(m, __uint_as_float(v.z), __uint_as_float(v.w));
     }
+    __device__ __forceinline__ void fold(const RawMax& o) { m = fmaxf(m, o.m); }
     __device__ __forceinline__ float value() const { return m; }
 };
 template <> struct RawMax<kBF16> {
@@ -480,6 +481,7 @@ template <> struct RawMax<kBF16> {
     __device__ __forceinline__ void fold(const uint4& v) {
         m = max_bf16x2(m, max_bf16x2(max_bf16x2(v.x, v.y), max_bf16x2(v.z, v.w)));
     }
+    __device__ __forceinline__ void fold(const RawMax& o) { m = max_bf16x2(m, o.m); }
     __device__ __forceinline__ float value() const {
         return fmaxf(__uint_as_float(m << 16), __uint_as_float(m & 0xffff0000u));
     }
@@ -611,11 +613,10 @@ struct LaneSpan {
     const uint4* src;
 };
 template <int DT>
-__device__ __forceinline__ LaneSpan lane_span(const RowGeom& g, int seg, int lane, int den = 1) {
+__device__ __forceinline__ LaneSpan lane_span(const RowGeom& g, int seg, int lane) {
     constexpr int EPV = ElemTraits<DT>::kEPV;
     int v_lo, v_hi;
     seg_range(g, seg, v_lo, v_hi);
-    if (den > 1) v_hi = min(v_hi, v_lo + (v_hi - v_lo + den - 1) / den);   // only the first 1/den of the segment
     const bool head_edge = g.pre > 0;
     const bool tail_edge = ((g.pre + g.V) % EPV) != 0;
     int i_lo = v_lo, i_hi = v_hi;

@@ -27,8 +27,10 @@ constexpr int kHistCopies = 8;           // interleaved copies of the histogram:
 constexpr float kMassScale = 1099511627776.0f;   // 2^40
 constexpr int kPoolCap = 2048;           // candidates of the whole cluster
 constexpr int kCandPerBlock = 1024;      // candidates one of several blocks may collect
-constexpr int kCounted = 256;            // up to this many group maxima or candidates are put in order by counting
+constexpr int kCounted = 256;            // up to this many candidates are put in order by counting
 constexpr int kMaxGroups = 2048;         // groups of threads whose maxima give the bound of a top-k
+constexpr int kOneWarp = 256;            // up to this many group maxima are searched by one warp
+constexpr int kStretches = 8;            // maxima that a thread keeps of the vectors it streams
 
 struct ThresholdArgs {
     const void* logits;
@@ -47,7 +49,7 @@ struct ThresholdArgs {
     float* entropy;          // [rows] out
     uint8_t* stop;           // [rows] out
     unsigned* status;        // device status word
-    int sample_den;          // candidate path: the first bound comes from 1/sample_den of every warp segment (1: all)
+    int groups;              // candidate path, top-k: log2 of the groups of threads per warp whose maxima bound the threshold
 };
 
 // Monotone image of a float: a < b  <=>  key(a) < key(b).  NaN counts as -inf.
@@ -107,8 +109,11 @@ enum : uint32_t {
 struct SelectShared {
     union {
         uint32_t priv[3][256][kHistCopies];   // count, mass low word, mass high word; per digit, per copy
-        Candidate landing[kPoolCap];          // candidate path, block 0: the peers' candidates, one region per block (the
+        struct {
+            Candidate landing[kPoolCap];      // candidate path, block 0: the peers' candidates, one region per block (the
                                               // candidates of a block alone)
+            uint16_t stretch_key[kStretches][kThreads];   // top-k, rows that do not fit the ring: see stream_maxima
+        };
     };
     union {
         alignas(16) float group_max[kMaxGroups];   // candidate path: group maxima of the whole cluster
@@ -121,7 +126,7 @@ struct SelectShared {
             uint32_t tot_cnt[256];            // the cluster's histogram
             unsigned long long tot_mass[256];
         };
-        uint32_t vec_list[kCandPerBlock];     // candidate path: vectors with an element at or above the bound
+        uint32_t vec_list[kCandPerBlock];     // candidate path: stretches (top-k) or vectors with an element at or above the bound
     };
     float blk_max;                        // this block's largest logit
     unsigned long long blk_above;         // this block's mass of the elements >= tau_k
@@ -134,17 +139,16 @@ struct SelectShared {
     unsigned long long bar_group;         // all group maxima have landed
     unsigned long long bar_pool;          // block 0: headers and candidates of all blocks have landed
     unsigned long long bar_verdict;       // the verdict has landed
-    uint32_t n_vec;                       // how many vectors are listed (may exceed the capacity)
+    uint32_t n_vec;                       // how many of these there are (may exceed the capacity)
     uint32_t n_cand;                      // how many candidates this block found (may exceed the capacity)
     uint32_t bound_key;                   // lower bound of the threshold
-    uint32_t better[kMaxCluster];         // ... and what each block makes of the candidates it has, if they do not fit
+    uint32_t better[kMaxCluster];         // ... and a better one that each block finds, if they do not fit
     uint32_t top_key;
+    int tied;                             // top-k: the bound is the largest group maximum, no better one exists
     // decision of a pass (written by warp 0)
     int bin;
     uint32_t cnt_above;
     unsigned long long mass_above;
-    unsigned long long mass_total;
-    unsigned long long mass_bin;
 };
 
 // Block 0's working set while it finishes a row from its candidates; lives in the streaming ring, free by then.
@@ -288,8 +292,8 @@ __device__ __forceinline__ void decide(SelectShared& sh, int lane, uint32_t k_re
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         const int bin = 255 - 8 * lane - j;
-        cn[j] = sh.tot_cnt[bin];
-        ms[j] = sh.tot_mass[bin];
+        cn[j] = kByMass ? 0u : sh.tot_cnt[bin];
+        ms[j] = kByMass ? sh.tot_mass[bin] : 0ull;
         csum += cn[j];
         msum += ms[j];
     }
@@ -297,15 +301,15 @@ __device__ __forceinline__ void decide(SelectShared& sh, int lane, uint32_t k_re
     unsigned long long minc = msum;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t cu = __shfl_up_sync(0xffffffffu, cinc, o);
-        const unsigned long long mu = shfl_up_u64(minc, o);
+        const uint32_t cu = kByMass ? 0u : __shfl_up_sync(0xffffffffu, cinc, o);
+        const unsigned long long mu = kByMass ? shfl_up_u64(minc, o) : 0ull;
         if (lane >= o) { cinc += cu; minc += mu; }
     }
     uint32_t cbefore = cinc - csum;              // digits above this lane's
     unsigned long long mbefore = minc - msum;
     int hit = -1;
     uint32_t c_at = 0;
-    unsigned long long m_at = 0, m_bin = 0;
+    unsigned long long m_at = 0;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         const bool reached = kByMass ? (mbefore + ms[j] >= p_rem) : (cbefore + cn[j] >= k_rem);
@@ -313,19 +317,16 @@ __device__ __forceinline__ void decide(SelectShared& sh, int lane, uint32_t k_re
             hit = 255 - 8 * lane - j;
             c_at = cbefore;
             m_at = mbefore;
-            m_bin = ms[j];
         }
         cbefore += cn[j];
         mbefore += ms[j];
     }
     const unsigned who = __ballot_sync(0xffffffffu, hit >= 0);
-    const unsigned long long total = __shfl_sync(0xffffffffu, static_cast<uint32_t>(minc), 31) |
-        (static_cast<unsigned long long>(__shfl_sync(0xffffffffu, static_cast<uint32_t>(minc >> 32), 31)) << 32);
     if (who == 0) {
         // nothing reaches the target (an empty histogram): stay at the lowest digit
-        if (lane == 0) { sh.bin = 0; sh.cnt_above = 0; sh.mass_above = 0; sh.mass_total = total; sh.mass_bin = 0; }
+        if (lane == 0) { sh.bin = 0; sh.cnt_above = 0; sh.mass_above = 0; }
     } else if (lane == __ffs(who) - 1) {
-        sh.bin = hit; sh.cnt_above = c_at; sh.mass_above = m_at; sh.mass_total = total; sh.mass_bin = m_bin;
+        sh.bin = hit; sh.cnt_above = c_at; sh.mass_above = m_at;
     }
 }
 
@@ -370,26 +371,31 @@ __device__ __forceinline__ unsigned long long mass_of_key(uint32_t key, float c,
 // ------------------------------------------------------------------ candidate path
 //
 // For a top-k with a small k (with or without the nucleus inside it) and for the nucleus alone: a lower bound t0 of
-// the threshold from one pass over the row, the elements >= t0 from a second one, everything else from these
-// candidates.
+// the threshold from one pass over the row, the elements >= t0 from what the pass has left in the ring or from a second look,
+// everything else from these candidates.
 //   top-k    the maxima of disjoint groups of threads are distinct elements of the row, so the k-th largest of them
-//            is a lower bound of tau_k.  With G groups about -G ln(1 - k/G) elements lie above it (G >= 2k: 1.4 k),
-//            so the groups are made as large as that allows, which keeps the exchange small.
+//            is a lower bound of tau_k.  With G groups about -G ln(1 - k/G) elements lie above it (G >= 1.5 k: 1.65 k),
+//            so the groups are made as large as that allows, which keeps the exchange and the search in it small.  The row
+//            is read once: of rows that do not fit the ring the maxima of stretches of vectors are kept, and only the
+//            stretches that reach the bound are fetched again.
 //   nucleus  elements of mass below (1 - top_p) Z / V weigh less than (1 - top_p) Z together, so none of them is
 //            in the nucleus, and neither with anything below Z in its place: the first pass takes maxima only, and the
 //            masses of the threads' maxima stand for Z.  The second pass also sums the masses of all elements, in fixed
 //            point and relative to the row's maximum, as the radix descent does: a cut must not depend on how many
 //            blocks share the row, nor on which way the row goes (with Z summed in fp32 it did, for running masses within
 //            1e-6 of top_p).
-// A segment that fits the ring (small launches) is still in shared memory for the second pass.  The blocks push
+// A segment that fits the ring (small launches) is still in shared memory for the second look.  The blocks push
 // their candidates into block 0 of the cluster, which puts up to kCounted of them in order by counting (several threads
 // per candidate) and finds tau_k, the nucleus cut and the sample by scans of one warp over the masses; in more these are
 // found by radix descents in shared memory.  It tells the other blocks whether they are needed again.  All
 // masses are 2^-40 fixed point, so nothing depends on the order in which they are added or candidates arrive.
-// Bound by the chain of exchanges for launches of up to about 100 rows, by the two passes over the row above that.
+// Bound by the chain of exchanges for launches of up to about 100 rows, by the pass (nucleus: the two passes) over the rows above
+// that.
 // Rows of 152064 bf16, top-k 50 + top-p 0.9, against cluster barriers with remote reads and a counting finish in every
 // block: draft step of 16 rows 18.3 -> 10.1 us, 64 rows 21.5 -> 14.3, 256 rows 41.0 -> 25.1; threshold of 2304 rows
-// 243 -> 174 us.  Top-p alone against the radix descent: 1040 rows 521 -> 91 us.
+// 243 -> 174 us.  Top-p alone against the radix descent: 1040 rows 521 -> 91 us.  A top-k that reads its rows once, with one
+// warp's search for the bound, against two passes (of launches above 48 MB one and a half) and counting: draft step of 32 such rows
+// 12.6 -> 10.0 us, threshold of 288 rows 24.4 -> 20.7, a round of 128 sequences of 256000 fp32, 3 draft steps, 319 -> 268.
 
 // Block-wide wait for an mbarrier of the exchange: one warp polls, the others sleep at the block barrier.
 __device__ __forceinline__ void bar_wait(unsigned long long& bar, uint32_t parity, unsigned* status, int tid) {
@@ -419,7 +425,7 @@ __device__ __forceinline__ uint32_t pool_select(SelectShared& sh, int n, uint32_
         if (kByMass) {
             for (int i = tid; i < 256 * kHistCopies; i += kThreads) { (&sh.priv[1][0][0])[i] = 0; (&sh.priv[2][0][0])[i] = 0; }
         }
-        if (tid < 256) { sh.tot_cnt[tid] = 0; sh.tot_mass[tid] = 0; }
+        if (!kByMass && tid < 256) sh.tot_cnt[tid] = 0;
         __syncthreads();
         for (int i = tid; i < n; i += kThreads) {
             const uint32_t key = key_of(i);
@@ -453,36 +459,36 @@ __device__ __forceinline__ uint32_t pool_select(SelectShared& sh, int n, uint32_
     return prefix;
 }
 
-// Leaves in sh.bound_key the k-th largest of the n values (as an order key), or somewhat less.  Few values by counting: it is
-// the smallest value with fewer than k values above it.  That is quadratic (2048 values: 190 us), so of more the upper 16 bits
-// are found by a descent and the others left zero.  Ends with a barrier.  (n <= kMaxGroups, a multiple of 16; 1 <= k <= n.)
-__device__ __forceinline__ void kth_largest(SelectShared& sh, int n, uint32_t k, int tid) {
-    if (n > kCounted) {
-        const auto key_of = [&](int i) { return order_key(sh.group_max[i]); };
-        const uint32_t key = pool_select<false>(sh, n, 0u, 32, 16, k, 0ull, tid, key_of, key_of);
-        if (tid == 0) sh.bound_key = key;
-        __syncthreads();
-        return;
+// A bound (as an order key) that at least k of n <= 32 * kPer values reach, n >= k >= 1, and not many more than k.  By one warp,
+// bit by bit below the bits that all of them share, the values in registers.  (Ranking all of them by comparing every pair in
+// all warps took 3200 cycles for 192 values in the kernel, two blocks on an SM; this 2100.)
+template <int kPer>
+__device__ __forceinline__ uint32_t kth_bound(const float* values, int n, uint32_t k, int lane, uint32_t& top) {
+    uint32_t key[kPer], low = 0xffffffffu;
+    top = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int i = lane + 32 * j;
+        key[j] = i < n ? order_key(values[i]) : 0u;
+        top = max(top, key[j]);
+        if (i < n) low = min(low, key[j]);
     }
-    const int shift = share_shift(n), per = 1 << shift, rows = kThreads >> shift;
-    const int sub = tid & (per - 1);
-    const float4* quads = reinterpret_cast<const float4*>(sh.group_max);
-    uint32_t best = 0xffffffffu;
-    for (int base = 0; base < n; base += rows) {
-        const int i = base + (tid >> shift);
-        const float v = i < n ? sh.group_max[i] : neg_inf();
-        uint32_t gt = 0;
-#pragma unroll 2
-        for (int q = sub; q < n / 4; q += per) {
-            const float4 w = quads[q];
-            gt += (w.x > v) + (w.y > v) + (w.z > v) + (w.w > v);
-        }
-        for (int o = per >> 1; o > 0; o >>= 1) gt += __shfl_xor_sync(0xffffffffu, gt, o);
-        if (i < n && gt < k) best = min(best, order_key(v));
+    top = __reduce_max_sync(0xffffffffu, top);
+    low = __reduce_min_sync(0xffffffffu, low);
+    if (top == low) return top;
+    uint32_t step = 0x80000000u >> __clz(top ^ low);      // the highest bit in which they differ: clear in the lowest
+    uint32_t bound = low & ~(2u * step - 1u);
+#pragma unroll 1
+    for (; step != 0; step >>= 1) {
+        const uint32_t pivot = bound | step;
+        uint32_t c = 0;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) c += __popc(__ballot_sync(0xffffffffu, key[j] >= pivot));
+        if (c < k) continue;
+        bound = pivot;
+        if (c <= k + k / 4) break;
     }
-    best = __reduce_min_sync(0xffffffffu, best);
-    if ((tid & 31) == 0) atomicMin(&sh.bound_key, best);
-    __syncthreads();
+    return bound;
 }
 
 __device__ __forceinline__ unsigned long long shfl_u64(unsigned long long v, int src) {
@@ -743,57 +749,197 @@ struct CollectInto {
     uint32_t vec_cap;
 };
 
-// Collects the elements >= t0v of the block's segments and (kMass) leaves the mass of all elements of every
-// warp's segment in sh.warp_above.  `resident`: every segment of the row fits the ring and lies there since pass 1 (a
-// property of the row, so the same in every warp: a block barrier depends on it).
-template <int DT, bool kMass>
-__device__ __forceinline__ void collect(const RowGeom& g, const LaneSpan& s, bool resident, uint32_t slot0, float t0v,
-                                        const CollectInto& to, SelectShared& sh, float c, float row_max) {
-    constexpr int EPV = ElemTraits<DT>::kEPV;
-    MassSum<DT> mass(c, row_max);
-    const bool lowest = !(t0v > neg_inf());      // no bound: every element, -inf and NaN (which counts as -inf) among them
-    auto place = [&](float x, uint32_t pos, int i) {
+// The elements of a row at or above a bound, as they are found.
+template <int DT>
+struct Collector {
+    static constexpr int EPV = ElemTraits<DT>::kEPV;
+    const RowGeom& g;
+    const CollectInto& to;
+    SelectShared& sh;
+    float bound;
+    bool lowest;      // no bound: every element, -inf and NaN (which counts as -inf) among them
+    __device__ __forceinline__ Collector(const RowGeom& g_, const CollectInto& to_, SelectShared& sh_, float bound_)
+        : g(g_), to(to_), sh(sh_), bound(bound_), lowest(!(bound_ > neg_inf())) {}
+    __device__ __forceinline__ bool above(float x) const { return x >= bound || lowest; }
+    __device__ __forceinline__ void place(float x, uint32_t pos, int i) const {
         if (pos < to.cap) to.cand[pos] = Candidate{order_key(x), static_cast<uint32_t>(i)};
-    };
+    }
     // A set that does not fit is of no use, and a flat row has tens of thousands of elements above the bound, each of which
     // would wait for its turn at the counter: collecting ends as soon as that is known, and a vector asks for all its places
     // at once (draft step with Gaussian logits, top-p 0.9: 1 row of 304 KB 39.3 -> 31.7 us, 384 rows of 64 KB 90 -> 70).
-    auto over = [&]() { return *static_cast<volatile uint32_t*>(&sh.n_cand) > to.cap; };
-    auto has = [&](const uint4& raw) {        // asked once per vector: it also counts its mass
-        RawMax<DT> m;
-        m.reset();
-        m.fold(raw);
-        const float top = m.value();
-        if (kMass) mass.vector(raw, top);
-        return top >= t0v || lowest;
-    };
-    auto visit = [&](const uint4& raw, int vi) {
+    __device__ __forceinline__ bool over() const { return *static_cast<volatile uint32_t*>(&sh.n_cand) > to.cap; }
+    __device__ __forceinline__ void visit(const uint4& raw, int vi) const {
         float x[EPV];
         ElemTraits<DT>::unpack(raw, x);
         uint32_t hits = 0;
 #pragma unroll
-        for (int j = 0; j < EPV; ++j) hits += x[j] >= t0v || lowest ? 1u : 0u;
+        for (int j = 0; j < EPV; ++j) hits += above(x[j]) ? 1u : 0u;
         if (hits == 0 || over()) return;
         uint32_t pos = atomicAdd(&sh.n_cand, hits);
 #pragma unroll
         for (int j = 0; j < EPV; ++j)
-            if (x[j] >= t0v || lowest) place(x[j], pos++, vi * EPV + j - g.pre);
-    };
-    auto edge = [&](int vi) {
+            if (above(x[j])) place(x[j], pos++, vi * EPV + j - g.pre);
+    }
+    // A vector that sticks out of the row; each(x) is told its elements.
+    template <class F>
+    __device__ __forceinline__ void edge(int vi, F&& each) const {
         float x[EPV];
         ElemTraits<DT>::unpack(ld_vec(g.base + vi), x);
 #pragma unroll
         for (int j = 0; j < EPV; ++j) {
             const int i = vi * EPV + j - g.pre;
             if (i < 0 || i >= g.V) continue;
-            if (kMass) mass.one(x[j]);
-            if (x[j] >= t0v || lowest) place(x[j], atomicAdd(&sh.n_cand, 1u), i);
+            each(x[j]);
+            if (above(x[j])) place(x[j], atomicAdd(&sh.n_cand, 1u), i);
         }
+    }
+};
+
+// How the vectors of a lane make up stretches, whose maxima are kept: `rounds` rounds of the ring (kStages vectors) each,
+// `count` of them (at most kStretches).
+struct Stretches {
+    int rounds, count;
+    __device__ __forceinline__ explicit Stretches(const RowGeom& g) {
+        const int all = ((g.vps + 31) / 32 + kStages - 1) / kStages;
+        rounds = (all + kStretches - 1) / kStretches;
+        count = (all + rounds - 1) / rounds;
+    }
+};
+
+// Pass 1 of a top-k: the largest logit of the thread's interior vectors.  Of rows that do not fit the ring, which would have
+// to be read again for the candidates, the maximum of every stretch of vectors is kept (the upper half of its order key);
+// only the few stretches that reach the bound are then fetched a second time, instead of the row.
+template <int DT>
+__device__ __forceinline__ float stream_maxima(const LaneSpan& s, uint32_t slot0, bool resident, const Stretches st,
+                                               uint16_t (*keys)[kThreads]) {
+    constexpr uint32_t kSlotStride = kThreads * 16;
+    RawMax<DT> all, part;
+    all.reset();
+    part.reset();
+    if (resident) {       // the vectors stay in the ring
+        stream_interior(s, slot0, [&](const uint4& raw, int) { all.fold(raw); });
+        return all.value();
+    }
+#pragma unroll
+    for (int k = 0; k < kStages; ++k) {
+        if (k < s.n) cp_async16(slot0 + k * kSlotStride, s.src + 32 * k);
+        cp_async_commit();
+    }
+    uint16_t* at = &keys[0][threadIdx.x];
+    int left = st.rounds;
+    const auto flush = [&]() {
+        *at = static_cast<uint16_t>(order_key(part.value()) >> 16);
+        at += kThreads;
+        all.fold(part);
+        part.reset();
+        left = st.rounds;
+    };
+    int it = 0;
+    for (; it + kStages <= s.n; it += kStages) {
+#pragma unroll
+        for (int k = 0; k < kStages; ++k) {
+            cp_async_wait<kStages - 1>();
+            const uint4 raw = lds128(slot0 + k * kSlotStride);
+            if (it + kStages + k < s.n) cp_async16(slot0 + k * kSlotStride, s.src + 32 * (it + kStages + k));
+            cp_async_commit();
+            part.fold(raw);
+        }
+        if (--left == 0) flush();
+    }
+    cp_async_wait<0>();
+    if (it < s.n || left < st.rounds) {
+        for (; it < s.n; ++it) part.fold(lds128(slot0 + (it & (kStages - 1)) * kSlotStride));
+        flush();
+    }
+    for (; at < &keys[st.count][0]; at += kThreads) *at = 0;       // a lane with fewer
+    return all.value();
+}
+
+// Pass 2 of a top-k: the elements at or above the bound (sh.bound_key).  `best`: what stream_maxima found.  `resident`: every
+// segment of the row fits the ring and lies there (a property of the row, so the same in every warp: a block barrier depends
+// on it).
+template <int DT>
+__device__ __forceinline__ void collect_top(const RowGeom& g, const LaneSpan& s, bool resident, const Stretches st, uint32_t slot0,
+                                            float best, int rank, const CollectInto& to, SelectShared& sh) {
+    const Collector<DT> c(g, to, sh, key_value(sh.bound_key));
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (resident) {
+        const unsigned hit = __ballot_sync(0xffffffffu, c.above(best));
+        if (__popc(hit) > 8) {      // gathered: every lane looks through its own vectors
+            revisit_interior(s, slot0, [&](const uint4& raw, int vi) { c.visit(raw, vi); }, [&]() { return c.over(); });
+        } else {
+            // the vectors of a lane that has something, side by side, four such lanes at a time
+            for (unsigned left = hit; left;) {
+                int src = -1;
+#pragma unroll
+                for (int q = 0; q < 32 / kStages; ++q) {
+                    if (q == lane / kStages) src = __ffs(left) - 1;
+                    left &= left - 1;
+                }
+                const int n = __shfl_sync(0xffffffffu, s.n, max(src, 0));
+                const int k = lane % kStages;
+                if (src >= 0 && k < n)
+                    c.visit(lds128(slot0 + (src - lane) * 16 + k * (kThreads * 16)), s.vi0 - lane + src + 32 * k);
+            }
+        }
+    } else {
+        const uint32_t cut = c.lowest ? 0u : sh.bound_key >> 16;
+        const int vectors = st.rounds * kStages;
+        for (int e = 0; e * vectors < s.n; ++e) {
+            if (sh.stretch_key[e][tid] < cut) continue;
+            const uint32_t pos = atomicAdd(&sh.n_vec, 1u);
+            if (pos < to.vec_cap) to.vec_list[pos] = static_cast<uint32_t>(e * kThreads + tid);
+        }
+        __syncthreads();
+        const uint32_t n_hit = sh.n_vec;
+        // kStages threads per stretch, which take its vectors in turn; two vectors of a thread under way at a time.  Of a set
+        // that does not fit, a top-k still wants as many as there is room for (see better_bound).
+        const uint32_t items = min(n_hit, to.vec_cap) * kStages;
+        for (int r = 0; r < st.rounds; ++r) {
+            const auto vector_of = [&](uint32_t i, LaneSpan& o) {      // which one of the lane's vectors, or -1
+                if (i >= items) return -1;
+                const uint32_t code = to.vec_list[i / kStages];
+                const int t = static_cast<int>(code % kThreads);
+                o = lane_span<DT>(g, rank * kWarps + (t >> 5), t & 31);
+                const int it = static_cast<int>(code / kThreads) * vectors + r * kStages + static_cast<int>(i % kStages);
+                return it < o.n ? it : -1;
+            };
+            for (uint32_t i = tid; i < items && !c.over(); i += 2 * kThreads) {
+                LaneSpan o0, o1;
+                const int it0 = vector_of(i, o0), it1 = vector_of(i + kThreads, o1);
+                uint4 raw0 = make_uint4(0, 0, 0, 0), raw1 = raw0;
+                if (it0 >= 0) raw0 = ld_vec(o0.src + 32 * it0);
+                if (it1 >= 0) raw1 = ld_vec(o1.src + 32 * it1);
+                if (it0 >= 0) c.visit(raw0, o0.vi0 + 32 * it0);
+                if (it1 >= 0) c.visit(raw1, o1.vi0 + 32 * it1);
+            }
+        }
+        if (n_hit > to.vec_cap) {
+            __syncthreads();
+            if (tid == 0) atomicAdd(&sh.n_cand, to.cap + 1);
+        }
+    }
+    if (s.head) c.edge(0, [](float) {});
+    if (s.tail) c.edge(g.nvec - 1, [](float) {});
+}
+
+// Pass 2 of the nucleus alone: the elements >= bound, and the mass of all elements of every warp's segment, which it leaves in
+// sh.warp_above.
+template <int DT>
+__device__ __forceinline__ void collect_mass(const RowGeom& g, const LaneSpan& s, bool resident, uint32_t slot0, float bound,
+                                             const CollectInto& to, SelectShared& sh, float scale, float row_max) {
+    const Collector<DT> c(g, to, sh, bound);
+    MassSum<DT> mass(scale, row_max);
+    auto has = [&](const uint4& raw) {        // asked once per vector: it also counts its mass
+        RawMax<DT> m;
+        m.reset();
+        m.fold(raw);
+        const float top = m.value();
+        mass.vector(raw, top);
+        return c.above(top);
     };
     if (resident) {
-        const auto look = [&](const uint4& raw, int vi) { if (has(raw)) visit(raw, vi); };
-        if constexpr (kMass) revisit_interior(s, slot0, look, over);
-        else revisit_interior(s, slot0, look);
+        revisit_interior(s, slot0, [&](const uint4& raw, int vi) { if (has(raw)) c.visit(raw, vi); }, [&]() { return c.over(); });
     } else {
         // the streaming loop only lists the vectors, which are few, and all threads look at them afterwards: with the
         // elements looked at inside the unrolled loop, 2304 rows of 304 KB took 272 us instead of 174
@@ -806,82 +952,111 @@ __device__ __forceinline__ void collect(const RowGeom& g, const LaneSpan& s, boo
         }, full);
         __syncthreads();
         const uint32_t nv = sh.n_vec;
-        // of a set that does not fit, a top-k still wants as many as there is room for (see candidate_path)
-        if (!kMass || nv <= to.vec_cap)
-            for (uint32_t i = threadIdx.x; i < min(nv, to.vec_cap); i += kThreads) visit(ld_vec(g.base + to.vec_list[i]), to.vec_list[i]);
-        if (nv > to.vec_cap) {
+        if (nv <= to.vec_cap) {
+            for (uint32_t i = threadIdx.x; i < nv; i += kThreads) c.visit(ld_vec(g.base + to.vec_list[i]), to.vec_list[i]);
+        } else {
             __syncthreads();
             if (threadIdx.x == 0) atomicAdd(&sh.n_cand, to.cap + 1);
         }
     }
-    if (s.head) edge(0);
-    if (s.tail) edge(g.nvec - 1);
-    if (kMass) {
-        const unsigned long long m = warp_scan_mass(mass.sum, threadIdx.x & 31);
-        if ((threadIdx.x & 31) == 31) sh.warp_above[threadIdx.x >> 5] = m;
-    }
+    if (s.head) c.edge(0, [&](float x) { mass.one(x); });
+    if (s.tail) c.edge(g.nvec - 1, [&](float x) { mass.one(x); });
+    const unsigned long long m = warp_scan_mass(mass.sum, threadIdx.x & 31);
+    if ((threadIdx.x & 31) == 31) sh.warp_above[threadIdx.x >> 5] = m;
 }
 
-// Groups of threads per warp whose maxima bound a top-k: a power of two, at least 2 k in the cluster if there are
-// that many threads (as a shift).
-__device__ __forceinline__ int group_shift(int S, int k) {
+// log2 of the groups of threads per warp whose maxima bound a top-k of a cluster of S blocks: at least 3/2 k groups in the
+// cluster, if there are that many threads.
+inline int choose_groups(int S, int k) {
     int g = 0;
-    while (g < 5 && (kWarps * S) << g < 2 * k) ++g;
-    return g;
-}
-// The largest number of groups, likewise.
-__device__ __forceinline__ int finest_groups(int S) {
-    int g = 0;
-    while (g < 5 && (kWarps * S) << (g + 1) <= kMaxGroups) ++g;
+    while (g < 5 && 2L * (kWarps * S << g) < 3L * k) ++g;
     return g;
 }
 
-// The k-th largest of the maxima of groups of threads, 2^shift groups a warp (`best` is the thread's maximum); the same in
-// every block.  The bar_group phase has been opened, in all blocks.
-__device__ __forceinline__ uint32_t group_bound(SelectShared& sh, float best, int shift, int S, int seg, int k, uint32_t phase,
-                                                unsigned* status, int tid) {
+// The k-th largest of the maxima of groups of threads, 2^shift groups a warp (`best` is the thread's maximum), or somewhat
+// less, left in sh.bound_key; the same in every block.  The first phase of bar_group has been opened, in all blocks.
+__device__ __forceinline__ void group_bound(SelectShared& sh, float best, int shift, int S, int seg, int k, unsigned* status, int tid) {
     const int lane = tid & 31, width = 32 >> shift;
     for (int o = width >> 1; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
     const int slot = (seg << shift) + (lane >> (5 - shift));
-    const bool leads = (lane & (width - 1)) == 0;
+    const int n = (kWarps * S) << shift;
+    const int first = lane & (width - 1);
     if (S == 1) {
-        if (leads) sh.group_max[slot] = best;
+        if (first == 0) sh.group_max[slot] = best;
         __syncthreads();
-    } else {
-        if (leads) {
-            for (int r = 0; r < S; ++r)
-                push4(map_to_rank(smem_addr(&sh.group_max[slot]), r), map_to_rank(smem_addr(&sh.bar_group), r),
-                      __float_as_uint(best));
-        }
-        bar_wait(sh.bar_group, phase, status, tid);
+    } else {      // the threads of a group share the blocks to send to
+        for (int r = first; r < S; r += width)
+            push4(map_to_rank(smem_addr(&sh.group_max[slot]), r), map_to_rank(smem_addr(&sh.bar_group), r), __float_as_uint(best));
+        if (tid < 32 && !mbar_wait_bounded(smem_addr(&sh.bar_group), 0) && tid == 0) atomicOr(status, SVIP_STATUS_WAIT_TIMEOUT);
+        if (n > kOneWarp) __syncthreads();
     }
-    kth_largest(sh, (kWarps * S) << shift, static_cast<uint32_t>(k), tid);
-    return sh.bound_key;
+    if (n > kOneWarp) {       // of many values the upper 16 bits of the bound, by a descent
+        const auto key_of = [&](int i) { return order_key(sh.group_max[i]); };
+        const uint32_t key = pool_select<false>(sh, n, 0u, 32, 16, static_cast<uint32_t>(k), 0ull, tid, key_of, key_of);
+        if (tid == 0) {
+            sh.bound_key = key;
+            sh.tied = 0;
+        }
+    } else if (tid < 32) {
+        uint32_t top;
+        const uint32_t key = n <= 128 ? kth_bound<4>(sh.group_max, n, static_cast<uint32_t>(k), lane, top)
+                                      : kth_bound<kOneWarp / 32>(sh.group_max, n, static_cast<uint32_t>(k), lane, top);
+        if (lane == 0) {
+            sh.bound_key = key;
+            sh.tied = key == top;
+        }
+    }
+    __syncthreads();
 }
 
-// A better bound for a top-k whose candidates do not fit.  The maxima of large groups bound next to nothing where the likely
-// tokens are gathered in few warps (a vocabulary in order of frequency), those of half of the row where they are in the
-// other half.  Either the maxima of the smallest groups (`finest` >= 0), or the k-th largest of what the blocks have stored,
-// which are elements of the row like any others.  Thresholds of rows of 50021 fp32 logits in order of frequency, top-k 50,
-// without and with the second attempt: 16 rows 29.6 and 18.0 us, 64 rows 39.9 and 22.1, 300 rows 123 and 42.  A function of
-// its own, because its code in line cost every top-k 3 %.
-__device__ __noinline__ uint32_t better_bound(SelectShared& sh, const Candidate* cand, uint32_t stored, float best, int finest, int S,
-                                              int rank, int k, unsigned* status) {
+// A better bound for a top-k whose candidates do not fit; the same in every block.  The maxima of large groups bound next to
+// nothing where the likely tokens are gathered in few warps (a vocabulary in order of frequency).  There every block that found
+// too many elements takes the maxima of its threads, or of their stretches of vectors, as groups, stores what reaches
+// the k-th largest of these (at least the first of them), and any block with k elements stored takes their k-th largest: a
+// bound for the row as well, and the blocks agree on the largest of these.  Rows of 50021 fp32 logits in order of frequency,
+// top-k 50, against the maxima of the smallest groups of the cluster (few rows) or the k-th largest of what happened to be
+// stored: 1 row 15.7 -> 13.3 us, 64 rows 22.4 -> 19.0, 300 rows 42.1 -> 36.6, 300 rows in reversed order 99.6 -> 35.9 (with
+// the descent in place of the second attempt 123).  A function of its own, because its code in line cost every top-k 3 %.
+template <int DT>
+__device__ __noinline__ uint32_t better_bound(SelectShared& sh, const CollectInto to, const RowGeom g, bool resident, uint32_t slot0,
+                                              float best, int S, int rank, int k, unsigned* status) {
     const int tid = threadIdx.x;
-    uint32_t bound = 0;
-    if (finest < 0 && stored >= static_cast<uint32_t>(k)) {
-        const auto key_of = [&](int i) { return cand[i].key; };
-        bound = pool_select<false>(sh, static_cast<int>(stored), 0u, 32, 16, static_cast<uint32_t>(k), 0ull, tid, key_of, key_of);
+    const uint32_t want = static_cast<uint32_t>(k);
+    const uint32_t found = sh.n_cand;
+    uint32_t bound = 0, stored = min(found, to.cap);
+    if (found > to.cap) {
+        const Stretches st(g);
+        const int groups = resident ? kThreads : st.count * kThreads;
+        if (resident) {
+            __syncthreads();
+            sh.group_max[tid] = best;       // where the candidates were
+            stored = 0;
+        }
+        __syncthreads();
+        if (groups >= k) {
+            const auto key_of = [&](int i) {
+                return resident ? order_key(sh.group_max[i]) : static_cast<uint32_t>((&sh.stretch_key[0][0])[i]) << 16;
+            };
+            bound = pool_select<false>(sh, groups, 0u, 32, 16, want, 0ull, tid, key_of, key_of);
+        }
+        if (bound > sh.bound_key) {
+            __syncthreads();
+            if (tid == 0) { sh.n_cand = 0; sh.n_vec = 0; sh.bound_key = bound; }
+            __syncthreads();
+            collect_top<DT>(g, lane_span<DT>(g, rank * kWarps + (tid >> 5), tid & 31), resident, st, slot0, best, rank, to, sh);
+            __syncthreads();
+            stored = min(sh.n_cand, to.cap);
+        }
+    }
+    if (stored >= want) {
+        const auto key_of = [&](int i) { return to.cand[i].key; };
+        bound = max(bound, pool_select<false>(sh, static_cast<int>(stored), 0u, 32, 16, want, 0ull, tid, key_of, key_of));
     }
     if (S > 1) {
         if (tid == 0) {
-            mbar_arrive_expect_tx(smem_addr(&sh.bar_group), static_cast<uint32_t>(finest < 0 ? S * 4 : (kWarps * S * 4) << finest));
+            mbar_arrive_expect_tx(smem_addr(&sh.bar_group), static_cast<uint32_t>(S * 4));
             if (rank != 0) mbar_arrive_expect_tx(smem_addr(&sh.bar_verdict), 16);
-            if (finest >= 0) sh.bound_key = 0xffffffffu;
         }
-        cluster_arrive();
-        cluster_wait();
-        if (finest >= 0) return group_bound(sh, best, finest, S, rank * kWarps + (tid >> 5), k, 1, status, tid);
         if (tid < S) push4(map_to_rank(smem_addr(&sh.better[rank]), tid), map_to_rank(smem_addr(&sh.bar_group), tid), bound);
         bar_wait(sh.bar_group, 1, status, tid);
         for (int r = 0; r < S; ++r) bound = max(bound, sh.better[r]);
@@ -890,20 +1065,19 @@ __device__ __noinline__ uint32_t better_bound(SelectShared& sh, const Candidate*
 }
 
 // Barriers and counters of the path; needs no global memory, so it runs before the predecessor has finished.
-__device__ __forceinline__ void candidate_open(SelectShared& sh, int S, int rank, int top_k, bool use_k, int tid) {
+__device__ __forceinline__ void candidate_open(SelectShared& sh, int S, int rank, int groups, bool use_k, int tid) {
     if (tid == 0) {
         if (S > 1) {
             mbar_init(smem_addr(&sh.ex.bar), 1);
             mbar_init(smem_addr(&sh.bar_group), 1);
             mbar_init(smem_addr(&sh.bar_verdict), 1);
             mbar_init(smem_addr(&sh.bar_pool), S);
-            if (use_k) mbar_arrive_expect_tx(smem_addr(&sh.bar_group), static_cast<uint32_t>((kWarps * S * 4) << group_shift(S, top_k)));
+            if (use_k) mbar_arrive_expect_tx(smem_addr(&sh.bar_group), static_cast<uint32_t>((kWarps * S * 4) << groups));
             else mbar_arrive_expect_tx(smem_addr(&sh.ex.bar), static_cast<uint32_t>(S * kWarps * sizeof(SegEntry)));
             if (rank != 0) mbar_arrive_expect_tx(smem_addr(&sh.bar_verdict), 16);   // block 0 gives the verdict
         }
         sh.n_cand = 0;
         sh.n_vec = 0;
-        sh.bound_key = 0xffffffffu;
     }
     if (S > 1) cluster_arrive_relaxed();     // the peers push only after their cluster_wait()
 }
@@ -923,23 +1097,26 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
     const CollectInto to = S == 1 ? CollectInto{sh.landing, kPoolCap, reinterpret_cast<uint32_t*>(sh.cand), 2 * kCandPerBlock}
                                   : CollectInto{sh.cand, kCandPerBlock, sh.vec_list, kCandPerBlock};
     const uint32_t region = kPoolCap / S;
-    const int gs = group_shift(S, a.top_k);
-    const int den = kTopK ? a.sample_den : 1;
+    const bool resident = g.vps <= 32 * kStages;
+    const Stretches stretches(g);
     // ---- pass 1: the largest logit of every thread, and from these the bound
-    const LaneSpan part = den > 1 ? lane_span<DT>(g, seg, lane, den) : span;
-    RawMax<DT> m;
-    m.reset();
-    stream_interior(part, slot0, [&](const uint4& raw, int) { m.fold(raw); });
-    float best = m.value();
-    if (part.head || part.tail) {
-        float x[EPV];
-        if (part.head) { unpack_masked<DT>(ld_vec(g.base), 0, g, x); best = fmaxf(best, vec_max<EPV>(x)); }
-        if (part.tail) { unpack_masked<DT>(ld_vec(g.base + g.nvec - 1), g.nvec - 1, g, x); best = fmaxf(best, vec_max<EPV>(x)); }
+    float best;
+    if constexpr (kTopK) {
+        best = stream_maxima<DT>(span, slot0, resident, stretches, sh.stretch_key);
+    } else {
+        RawMax<DT> m;
+        m.reset();
+        stream_interior(span, slot0, [&](const uint4& raw, int) { m.fold(raw); });
+        best = m.value();
     }
-    uint32_t first_bound = 0;
+    if (span.head || span.tail) {
+        float x[EPV];
+        if (span.head) { unpack_masked<DT>(ld_vec(g.base), 0, g, x); best = fmaxf(best, vec_max<EPV>(x)); }
+        if (span.tail) { unpack_masked<DT>(ld_vec(g.base + g.nvec - 1), g.nvec - 1, g, x); best = fmaxf(best, vec_max<EPV>(x)); }
+    }
     if constexpr (kTopK) {
         if (S > 1) cluster_wait();
-        first_bound = group_bound(sh, best, gs, S, seg, a.top_k, 0, a.status, tid);
+        group_bound(sh, best, a.groups, S, seg, a.top_k, a.status, tid);
     } else {
         Partial t;
         t.m = warp_max(best); t.idx = kIntMax; t.A = 0.f;
@@ -950,30 +1127,31 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
         } else {
             cluster_wait();
             exchange_send(sh.ex, S, rank, warp, lane, t);
-            bar_wait(sh.ex.bar, 0, a.status, tid);
         }
-        // every warp forms the same sums from the same entries
-        const Partial r = merge_entries<1>(LocalSegments{sh.ex.all}, S * kWarps, a.c, lane);
-        row_max = r.m;       // what the radix descent needs first
-        if (!(fabsf(r.m) <= kMaxLogit) || !(r.Z > 0.f)) return kVerdictDescend;   // in every block alike
-        // no element weighs more than 1, so the nucleus has at least top_p Z of them: a flat row does not fit
-        if (a.top_p * r.Z > static_cast<float>(kPoolCap)) return kVerdictDescend;
-        // in log2 units, a little low for the roundings of the weights, and of the bound as a logit
-        const float cut = log2f((1.f - a.top_p) * r.Z / static_cast<float>(g.V)) - 0.05f;
-        if (tid == 0) sh.bound_key = order_key((__fmul_rn(r.m, a.c) + cut) / a.c - 5e-7f * fabsf(r.m));
+        if (warp == 0) {       // one warp: in all of them these steps would get in each other's way
+            if (S > 1 && !mbar_wait_bounded(smem_addr(&sh.ex.bar), 0) && lane == 0) atomicOr(a.status, SVIP_STATUS_WAIT_TIMEOUT);
+            const Partial r = merge_entries<1>(LocalSegments{sh.ex.all}, S * kWarps, a.c, lane);
+            // no element weighs more than 1, so the nucleus has at least top_p Z of them: a flat row does not fit
+            const bool fits = fabsf(r.m) <= kMaxLogit && r.Z > 0.f && a.top_p * r.Z <= static_cast<float>(kPoolCap);
+            // in log2 units, a little low for the roundings of the weights, and of the bound as a logit
+            const float cut = log2f((1.f - a.top_p) * r.Z / static_cast<float>(g.V)) - 0.05f;
+            if (lane == 0) {
+                sh.blk_max = r.m;
+                sh.bin = fits;
+                sh.bound_key = order_key((__fmul_rn(r.m, a.c) + cut) / a.c - 5e-7f * fabsf(r.m));
+            }
+        }
         __syncthreads();
+        row_max = sh.blk_max;       // what the radix descent needs first
+        if (!sh.bin) return kVerdictDescend;   // in every block alike
     }
-    // Whether smaller groups are worth a second attempt: if all likely tokens are gathered in as few warps as can hold them, the
-    // candidates fit a block all the same.
-    const int finest = finest_groups(S);
-    const bool finer = S > 1 && den == 1 && finest > gs && (static_cast<long>(a.top_k) * g.vps * EPV >> finest) <= 3 * kCandPerBlock / 2;
     uint32_t parity = 0;
     for (;;) {
         // ---- pass 2: the candidates
-        const float t0v = key_value(sh.bound_key);
         pdl_launch_dependents();
-        const bool resident = den == 1 && g.vps <= 32 * kStages;
-        collect<DT, !kTopK>(g, span, resident, slot0, t0v, to, sh, a.c, row_max);
+        const uint32_t bound = sh.bound_key;
+        if constexpr (kTopK) collect_top<DT>(g, span, resident, stretches, slot0, best, rank, to, sh);
+        else collect_mass<DT>(g, span, resident, slot0, key_value(bound), to, sh, a.c, row_max);
         __syncthreads();
         uint32_t verdict;
         const uint32_t mine = sh.n_cand;
@@ -1019,7 +1197,7 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
             const uint32_t total = __shfl_sync(0xffffffffu, end, kMaxCluster - 1);
             const bool fits = !__any_sync(0xffffffffu, count > to.cap) && total <= kPoolCap;
             if (!fits || total < static_cast<uint32_t>(kTopK ? a.top_k : 1)) {
-                verdict = kTopK && !fits && parity == 0 && (S == 1 || den > 1 || finer) ? kVerdictRetry : kVerdictDescend;
+                verdict = kTopK && !fits && parity == 0 && !sh.tied ? kVerdictRetry : kVerdictDescend;
                 tell(verdict, 0u);
             } else {
                 // two warps copy the candidates of each block
@@ -1042,13 +1220,13 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
         // ---- once more with a better bound
         __syncthreads();
         parity = 1;
-        const uint32_t bound = better_bound(sh, to.cand, min(mine, to.cap), best, finer ? finest : -1, S, rank, a.top_k, a.status);
-        if (bound <= first_bound) return kVerdictDescend;      // in every block alike
+        const uint32_t better = better_bound<DT>(sh, to, g, resident, slot0, best, S, rank, a.top_k, a.status);
+        if (better <= bound) return kVerdictDescend;      // in every block alike
         __syncthreads();
         if (tid == 0) {
             sh.n_cand = 0;
             sh.n_vec = 0;
-            sh.bound_key = bound;
+            sh.bound_key = better;
         }
         __syncthreads();
     }
@@ -1091,7 +1269,7 @@ __global__ void __launch_bounds__(kThreads, 2) row_threshold_kernel(ThresholdArg
     // a small k against the number of threads of the cluster, or the nucleus alone: two passes over the row
     const bool by_candidates = kTopK ? a.top_k <= (S * kThreads) / 4 : use_p;
     const LaneSpan span = lane_span<DT>(g, rank * kWarps + warp, lane);
-    if (by_candidates) candidate_open(sh, S, rank, a.top_k, kTopK, tid);
+    if (by_candidates) candidate_open(sh, S, rank, a.groups, kTopK, tid);
     if (!a.active && lane == 0) prefetch_segment(g, rank * kWarps + warp, kRingBytes / kWarps);
     pdl_wait();
     if (kDraft && a.active && !a.active[row]) {         // the whole cluster leaves together
