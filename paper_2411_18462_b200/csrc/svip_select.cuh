@@ -27,9 +27,9 @@ constexpr int kHistCopies = 8;           // interleaved copies of the histogram:
 constexpr float kMassScale = 1099511627776.0f;   // 2^40
 constexpr int kPoolCap = 2048;           // candidates of the whole cluster
 constexpr int kCandPerBlock = 1024;      // candidates one of several blocks may collect
-constexpr int kCounted = 256;            // up to this many candidates are put in order by counting
+constexpr int kSorted = 256;             // up to this many candidates are put in order, the keys by one warp
 constexpr int kMaxGroups = 2048;         // groups of threads whose maxima give the bound of a top-k
-constexpr int kOneWarp = 256;            // up to this many group maxima are searched by one warp
+constexpr int kOneWarp = 512;            // up to this many group maxima are searched by one warp
 constexpr int kStretches = 8;            // maxima that a thread keeps of the vectors it streams
 
 struct ThresholdArgs {
@@ -155,11 +155,11 @@ struct SelectShared {
 struct PoolScratch {
     Candidate pool[kPoolCap];
     union {
-        struct {                                         // up to kCounted candidates
-            uint32_t key_desc[kCounted];                 // keys from the largest down ...
-            unsigned long long mass_desc[kCounted];      // ... and their masses
-            Candidate by_idx[kCounted];                  // candidates in index order ...
-            unsigned long long mass_idx[kCounted];       // ... and their masses
+        struct {                                         // up to kSorted candidates
+            Candidate by_idx[kSorted];                   // candidates in index order ...
+            unsigned long long mass_idx[kSorted];        // ... and their masses
+            uint32_t key_t;                              // key of the threshold
+            int unusable;                                // no finite mass in the row
         };
         unsigned long long mass[kPoolCap];               // more: the masses of the pool
     };
@@ -363,9 +363,12 @@ __device__ __forceinline__ float2 kept_stats(float row_max, unsigned long long k
     return make_float2(row_max, finite ? static_cast<float>(static_cast<double>(kept_mass) / 1099511627776.0) : 0.f);
 }
 
+__device__ __forceinline__ float weight_of_key(uint32_t key, float c, float M) {
+    return ex2_approx(fmaxf(__fmaf_rn(key_value(key), c, -M), kArgFloor));
+}
+__device__ __forceinline__ unsigned long long mass_of_weight(float w) { return __float2ull_rz(w * kMassScale); }
 __device__ __forceinline__ unsigned long long mass_of_key(uint32_t key, float c, float M) {
-    const float w = ex2_approx(fmaxf(__fmaf_rn(key_value(key), c, -M), kArgFloor));
-    return __float2ull_rz(w * kMassScale);
+    return mass_of_weight(weight_of_key(key, c, M));
 }
 
 // ------------------------------------------------------------------ candidate path
@@ -385,9 +388,8 @@ __device__ __forceinline__ unsigned long long mass_of_key(uint32_t key, float c,
 //            blocks share the row, nor on which way the row goes (with Z summed in fp32 it did, for running masses within
 //            1e-6 of top_p).
 // A segment that fits the ring (small launches) is still in shared memory for the second look.  The blocks push
-// their candidates into block 0 of the cluster, which puts up to kCounted of them in order by counting (several threads
-// per candidate) and finds tau_k, the nucleus cut and the sample by scans of one warp over the masses; in more these are
-// found by radix descents in shared memory.  It tells the other blocks whether they are needed again.  All
+// their candidates into block 0 of the cluster, which puts up to kSorted of them in order and finds tau_k, the nucleus cut and
+// the sample by scans of one warp over the masses; in more these are found by radix descents in shared memory.  It tells the other blocks whether they are needed again.  All
 // masses are 2^-40 fixed point, so nothing depends on the order in which they are added or candidates arrive.
 // Bound by the chain of exchanges for launches of up to about 100 rows, by the pass (nucleus: the two passes) over the rows above
 // that.
@@ -401,13 +403,6 @@ __device__ __forceinline__ unsigned long long mass_of_key(uint32_t key, float c,
 __device__ __forceinline__ void bar_wait(unsigned long long& bar, uint32_t parity, unsigned* status, int tid) {
     if (tid < 32 && !mbar_wait_bounded(smem_addr(&bar), parity) && tid == 0) atomicOr(status, SVIP_STATUS_WAIT_TIMEOUT);
     __syncthreads();
-}
-
-// log2 of how many threads (a power of two, at most 32) can share each of n items in one pass of the block.
-__device__ __forceinline__ int share_shift(int n) {
-    int k = 0;
-    while (k < 5 && (2 * n) << k <= kThreads) ++k;
-    return k;
 }
 
 // Radix descent over n items of shared memory in bits [low, high) of their keys, at most 8 bits a level; `prefix` holds the
@@ -461,7 +456,7 @@ __device__ __forceinline__ uint32_t pool_select(SelectShared& sh, int n, uint32_
 
 // A bound (as an order key) that at least k of n <= 32 * kPer values reach, n >= k >= 1, and not many more than k.  By one warp,
 // bit by bit below the bits that all of them share, the values in registers.  (Ranking all of them by comparing every pair in
-// all warps took 3200 cycles for 192 values in the kernel, two blocks on an SM; this 2100.)
+// all warps took 3200 cycles for 192 values in the kernel, two blocks on an SM; this 1000 for 96.)
 template <int kPer>
 __device__ __forceinline__ uint32_t kth_bound(const float* values, int n, uint32_t k, int lane, uint32_t& top) {
     uint32_t key[kPer], low = 0xffffffffu;
@@ -483,10 +478,11 @@ __device__ __forceinline__ uint32_t kth_bound(const float* values, int n, uint32
         const uint32_t pivot = bound | step;
         uint32_t c = 0;
 #pragma unroll
-        for (int j = 0; j < kPer; ++j) c += __popc(__ballot_sync(0xffffffffu, key[j] >= pivot));
+        for (int j = 0; j < kPer; ++j) c += key[j] >= pivot ? 1u : 0u;
+        c = __reduce_add_sync(0xffffffffu, c);
         if (c < k) continue;
         bound = pivot;
-        if (c <= k + k / 4) break;
+        if (c <= k + k / 8) break;
     }
     return bound;
 }
@@ -504,69 +500,125 @@ __device__ __forceinline__ unsigned long long nucleus_target(float top_p, unsign
     return want > total ? total : want;
 }
 
-// Block 0, warp 0: threshold, statistics and (kDraft) the sample from n <= kCounted candidates, in order both ways
-// in `ps`.  Lane l owns the positions [l * per, (l + 1) * per) of both orders.  row_mass: mass of the whole row
-// (nucleus alone).  `finite` is false for a row whose maximum is not a number the masses can be taken against.
-template <bool kDraft, bool kTopK>
-__device__ __forceinline__ void finish_sorted(const PoolScratch& ps, int n, const ThresholdArgs& a, bool use_p,
-                                              unsigned long long row_mass, float row_max, float M, bool finite, int row,
-                                              int lane) {
-    const int per = (n + 31) / 32;
-    const int lo = min(lane * per, n), hi = min(lo + per, n);
-    unsigned long long sum = 0;
-    for (int i = lo; i < hi; ++i) sum += ps.mass_desc[i];
-    const unsigned long long before = warp_scan_mass(sum, lane) - sum;
-    uint32_t key_t = kTopK ? ps.key_desc[a.top_k - 1] : 0u;
-    if (use_p && finite) {
-        unsigned long long zk = row_mass;
-        if (kTopK) {      // mass of the candidates >= tau_k
-            zk = 0;
-            for (int i = lo; i < hi; ++i)
-                if (ps.key_desc[i] >= key_t) zk += ps.mass_desc[i];
-            zk = shfl_u64(warp_scan_mass(zk, lane), 31);
+// Sums over the lanes of a warp of integers below 2^48 in magnitude: 24 bits and the rest are summed apart, in 32 bits each, which
+// takes no carries and half the instructions.
+__device__ __forceinline__ unsigned long long warp_total_mass(unsigned long long v) {
+    const uint32_t lo = __reduce_add_sync(0xffffffffu, static_cast<uint32_t>(v) & 0xffffffu);
+    const uint32_t hi = __reduce_add_sync(0xffffffffu, static_cast<uint32_t>(v >> 24));
+    return (static_cast<unsigned long long>(hi) << 24) + lo;
+}
+__device__ __forceinline__ long long warp_total_signed(long long v) {
+    const uint32_t lo = __reduce_add_sync(0xffffffffu, static_cast<uint32_t>(v) & 0xffffffu);
+    const int hi = __reduce_add_sync(0xffffffffu, static_cast<int>(v >> 24));
+    return static_cast<long long>(hi) * (1 << 24) + lo;
+}
+__device__ __forceinline__ unsigned long long warp_prefix_mass(unsigned long long v, int lane) {     // inclusive
+    uint32_t lo = static_cast<uint32_t>(v) & 0xffffffu, hi = static_cast<uint32_t>(v >> 24);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t l = __shfl_up_sync(0xffffffffu, lo, o), h = __shfl_up_sync(0xffffffffu, hi, o);
+        if (lane >= o) { lo += l; hi += h; }
+    }
+    return (static_cast<unsigned long long>(hi) << 24) + lo;
+}
+
+// A block barrier that the warps may reach in different places of the code.
+__device__ __forceinline__ void block_meet() { asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory"); }
+
+// Sorts the 32 * kPer keys of a warp from the largest down (bitonic network); lane l ends up with places l * kPer ....
+template <int kPer>
+__device__ __forceinline__ void sort_down(uint32_t (&key)[kPer], int lane) {
+#pragma unroll
+    for (int size = 2; size <= 32 * kPer; size <<= 1) {
+#pragma unroll
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) {
+                const bool down = ((lane * kPer + j) & size) == 0;
+                if (stride >= kPer) {
+                    const uint32_t other = __shfl_xor_sync(0xffffffffu, key[j], stride / kPer);
+                    key[j] = ((lane & (stride / kPer)) == 0) == down ? max(key[j], other) : min(key[j], other);
+                } else if ((j & stride) == 0) {
+                    const uint32_t hi = max(key[j], key[j | stride]), lo = min(key[j], key[j | stride]);
+                    key[j] = down ? hi : lo;
+                    key[j | stride] = down ? lo : hi;
+                }
+            }
         }
+    }
+}
+
+// Block 0, warp 0: the threshold of a row from its n <= 32 * kPer candidates in order of their keys, which stay in registers, the
+// statistics, and (kDraft) the entropy; the sample waits at the block barrier for the threshold, which is left in ps.key_t.
+// row_mass: mass of the whole row (nucleus alone).  A row whose maximum is not a number that masses can be taken against gets,
+// in a draft step, a threshold only.
+template <bool kDraft, bool kTopK, int kPer, class Tell>
+__device__ __forceinline__ void finish_by_key(PoolScratch& ps, int n, const ThresholdArgs& a, bool use_p, unsigned long long row_mass,
+                                              int row, int lane, Tell&& tell) {
+    uint32_t key[kPer];
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) key[j] = lane + 32 * j < n ? ps.pool[lane + 32 * j].key : 0u;
+    sort_down<kPer>(key, lane);
+    const float row_max = key_value(__shfl_sync(0xffffffffu, key[0], 0));      // the largest candidate is the largest logit of the row
+    const bool finite = fabsf(row_max) <= kMaxLogit;
+    const float M = finite ? __fmul_rn(row_max, a.c) : 0.f;
+    if (!kDraft || finite) tell(kVerdictDone, 0u);
+    uint32_t key_t = 0;
+    if (kTopK) {
+#pragma unroll
+        for (int j = 0; j < kPer; ++j)
+            if ((a.top_k - 1) % kPer == j) key_t = key[j];
+        key_t = __shfl_sync(0xffffffffu, key_t, (a.top_k - 1) / kPer);
+    }
+    float w[kPer];       // the masses, before their conversion: half the registers
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) w[j] = key[j] ? weight_of_key(key[j], a.c, M) : 0.f;
+    if (use_p && finite) {
+        unsigned long long sum = 0, kept = 0;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const unsigned long long m = mass_of_weight(w[j]);
+            sum += m;
+            if (kTopK && key[j] >= key_t) kept += m;
+        }
+        const unsigned long long zk = kTopK ? warp_total_mass(kept) : row_mass;     // kTopK: of the candidates >= tau_k
+        const unsigned long long incl = warp_prefix_mass(sum, lane);
         if (zk > 0) {
             const unsigned long long want = nucleus_target(a.top_p, zk);
-            unsigned long long cum = before;
-            int at = kIntMax;
-            for (int i = lo; i < hi; ++i) {
-                cum += ps.mass_desc[i];
-                if (cum >= want && at == kIntMax) at = i;
+            unsigned long long cum = incl - sum;
+            uint32_t at = 0, last = 0xffffffffu;       // key at which the sum is reached; lowest key
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) {
+                cum += mass_of_weight(w[j]);
+                if (cum >= want) at = max(at, key[j]);
+                if (key[j]) last = key[j];
             }
-            at = warp_min_int(at);
-            if (at == kIntMax) at = n - 1;         // rounding at the very end of the candidates: all of them
-            key_t = max(key_t, ps.key_desc[at]);
+            const unsigned who = __ballot_sync(0xffffffffu, incl >= want);
+            if (who) at = __shfl_sync(0xffffffffu, at, __ffs(who) - 1);
+            else at = __reduce_min_sync(0xffffffffu, last);      // rounding at the very end of the candidates: all of them
+            key_t = max(key_t, at);
         }
     }
     if (lane == 0) a.thr[row] = key_t ? key_value(key_t) : neg_inf();
-    if (!a.stats && !kDraft) return;
-    // kept candidates in index order
-    unsigned long long zi = 0;
-    long long term = 0;
-    for (int i = lo; i < hi; ++i) {
-        if (ps.by_idx[i].key < key_t) continue;
-        zi += ps.mass_idx[i];
-        if (kDraft) {
-            const float arg = fmaxf(__fmaf_rn(key_value(ps.by_idx[i].key), a.c, -M), kArgFloor);
-            term += __float2ll_rz(ex2_approx(arg) * arg * kMassScale);
-        }
+    if (kDraft) {
+        if (lane == 0) { ps.key_t = key_t; ps.unusable = !finite; }
+        block_meet();
+        if (!finite) return;
+    } else if (!a.stats) {
+        return;
     }
-    const unsigned long long incl = warp_scan_mass(zi, lane);
-    const unsigned long long zt = shfl_u64(incl, 31);
+    unsigned long long z = 0;
+    long long term = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        if (key[j] < key_t || key[j] == 0) continue;
+        z += mass_of_weight(w[j]);
+        if (kDraft) term += __float2ll_rz(w[j] * fmaxf(__fmaf_rn(key_value(key[j]), a.c, -M), kArgFloor) * kMassScale);
+    }
+    const unsigned long long zt = warp_total_mass(z);
     if (lane == 0 && a.stats) a.stats[row] = kept_stats(row_max, zt, finite);
     if (!kDraft) return;
-    const long long aq = static_cast<long long>(shfl_u64(warp_scan_mass(static_cast<unsigned long long>(term), lane), 31));
-    const float u = a.uniforms[row];
-    const unsigned long long target = static_cast<unsigned long long>(static_cast<double>(u) * static_cast<double>(zt));
-    unsigned long long cum = incl - zi;
-    int token = -1;
-    for (int i = lo; i < hi; ++i) {
-        if (ps.by_idx[i].key < key_t) continue;
-        const unsigned long long next = cum + ps.mass_idx[i];
-        if (cum <= target && target < next) token = static_cast<int>(ps.by_idx[i].idx);
-        cum = next;
-    }
-    if (token >= 0) a.token[row] = token;      // exactly one lane: target < zt
+    const long long aq = warp_total_signed(term);
     if (lane == 0) {
         const float Z = static_cast<float>(static_cast<double>(zt) / 1099511627776.0);
         const float A = static_cast<float>(static_cast<double>(aq) / 1099511627776.0);
@@ -576,50 +628,74 @@ __device__ __forceinline__ void finish_sorted(const PoolScratch& ps, int n, cons
     }
 }
 
+// Block 0, one warp: the sample from n <= kSorted candidates in index order, of which those with a key >= key_t are kept.  Lane l
+// owns the places [l * per, (l + 1) * per).
+__device__ __forceinline__ void sample_by_index(const PoolScratch& ps, int n, uint32_t key_t, float u, int32_t* token, int lane) {
+    constexpr int kPer = kSorted / 32;
+    const int per = (n + 31) / 32;
+    const int lo = lane * per;
+    const int mine = max(0, min(per, n - lo));
+    unsigned long long sum = 0, cum[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        if (k < mine && ps.by_idx[lo + k].key >= key_t) sum += ps.mass_idx[lo + k];
+        cum[k] = sum;
+    }
+    const unsigned long long incl = warp_prefix_mass(sum, lane), before = incl - sum;
+    const unsigned long long target = static_cast<unsigned long long>(static_cast<double>(u) * static_cast<double>(shfl_u64(incl, 31)));
+    if (before <= target && target < incl) {      // exactly one lane: the target is less than the total
+        int at = lo;
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) at += k < mine && before + cum[k] <= target ? 1 : 0;
+        *token = static_cast<int32_t>(ps.by_idx[at].idx);
+    }
+}
+
 // Block 0 with all candidates of the cluster in ps.pool: finds the threshold and writes what it can.  Returns the
 // verdict for the row (kVerdictDone, or kVerdictStream when the draft step has to be streamed at key_out), which
-// `tell` passes on to the other blocks as soon as it is certain.
+// `tell` passes on to the other blocks as soon as it is certain.  A chain of dependent steps.  Up to kSorted candidates: warp 0
+// sorts the keys in registers and finds the threshold while the others put the candidates in index order by counting (80
+// candidates: 3300 cycles for both orders by counting in all warps and 5200 for the rest in one warp that read its places anew in
+// every step; 3200 in all now.  Draft step of 32 rows of 304 KB, top-k 50 + top-p 0.9, 10.0 -> 8.0 us, 8 rows of 64 KB fp32 8.6 -> 7.2).
 template <int DT, bool kDraft, bool kTopK, class Tell>
 __device__ __forceinline__ uint32_t finish_pool(SelectShared& sh, PoolScratch& ps, int n, const ThresholdArgs& a, bool use_p,
                                                 unsigned long long row_mass, int row, int tid,
                                                 uint32_t& key_out, Tell&& tell) {
     const int lane = tid & 31, warp = tid >> 5;
-    if (n <= kCounted) {
-        // position of every candidate in both orders, by counting; `per` threads share a candidate
-        const int shift = share_shift(n), per = 1 << shift;
-        const int sub = tid & (per - 1), i = tid >> shift;
-        const Candidate me = i < n ? ps.pool[i] : Candidate{0u, 0u};
-        uint32_t above = 0, left = 0, top = 0;
+    if (n <= kSorted) {
+        uint32_t verdict = kVerdictDone;
+        if (warp == 0) {
+            if (n <= 64) finish_by_key<kDraft, kTopK, 2>(ps, n, a, use_p, row_mass, row, lane, tell);
+            else if (n <= 128) finish_by_key<kDraft, kTopK, 4>(ps, n, a, use_p, row_mass, row, lane, tell);
+            else finish_by_key<kDraft, kTopK, kSorted / 32>(ps, n, a, use_p, row_mass, row, lane, tell);
+        } else if (kDraft) {
+            const float u = warp == 1 ? a.uniforms[row] : 0.f;
+            const int i = (warp - 1) * 32 + lane;
+            if (i - lane < n) {
+                const Candidate me = i < n ? ps.pool[i] : Candidate{0u, 0u};
+                const uint4* pairs = reinterpret_cast<const uint4*>(ps.pool);      // the one behind the last is a stand-in if n is odd
+                uint32_t top = 0;
+                int left = 0, left2 = 0;
 #pragma unroll 4
-        for (int j = sub; j < n; j += per) {
-            const Candidate o = ps.pool[j];
-            above += (o.key > me.key || (o.key == me.key && o.idx < me.idx)) ? 1u : 0u;
-            left += o.idx < me.idx ? 1u : 0u;
-            top = max(top, o.key);
+                for (int j = 0; j < (n + 1) / 2; ++j) {
+                    const uint4 o = pairs[j];
+                    left += o.y < me.idx ? 1 : 0;
+                    left2 += o.w < me.idx ? 1 : 0;
+                    top = max(top, max(o.x, o.z));
+                }
+                if (i < n) {
+                    const float row_max = key_value(top);
+                    ps.by_idx[left + left2] = me;
+                    ps.mass_idx[left + left2] = mass_of_key(me.key, a.c, fabsf(row_max) <= kMaxLogit ? __fmul_rn(row_max, a.c) : 0.f);
+                }
+            }
+            block_meet();
+            if (warp == 1 && !ps.unusable) sample_by_index(ps, n, ps.key_t, u, a.token + row, lane);
         }
-        for (int o = per / 2; o > 0; o >>= 1) {
-            above += __shfl_xor_sync(0xffffffffu, above, o);
-            left += __shfl_xor_sync(0xffffffffu, left, o);
-        }
-        top = __reduce_max_sync(0xffffffffu, top);     // every candidate is seen by some lane of the warp, whatever `per`
-        const float row_max = key_value(top);          // the largest candidate is the largest logit of the row
-        const bool finite = fabsf(row_max) <= kMaxLogit;
-        const float M = finite ? __fmul_rn(row_max, a.c) : 0.f;
-        const uint32_t verdict = kDraft && !finite ? kVerdictStream : kVerdictDone;
-        if (i < n && sub == 0) {
-            const unsigned long long w = mass_of_key(me.key, a.c, M);
-            ps.key_desc[above] = me.key;
-            ps.mass_desc[above] = w;
-            ps.by_idx[left] = me;
-            ps.mass_idx[left] = w;
-        }
-        __syncthreads();
-        key_out = kTopK ? ps.key_desc[a.top_k - 1] : 0u;   // what a row without finite mass is cut at
-        tell(verdict, key_out);
+        if (kDraft && ps.unusable) verdict = kVerdictStream;
         if (verdict == kVerdictStream) {
-            if (tid == 0) a.thr[row] = key_out ? key_value(key_out) : neg_inf();
-        } else if (warp == 0) {
-            finish_sorted<kDraft, kTopK>(ps, n, a, use_p, row_mass, row_max, M, finite, row, lane);
+            key_out = ps.key_t;                        // what a row without finite mass is cut at
+            if (warp == 0) tell(verdict, key_out);
         }
         return verdict;
     }
@@ -749,6 +825,14 @@ struct CollectInto {
     uint32_t vec_cap;
 };
 
+// Element j of a vector.
+template <int DT>
+__device__ __forceinline__ float pick_element(const uint4& v, int j) {
+    const int w = DT == kBF16 ? j >> 1 : j;
+    const uint32_t word = w & 2 ? (w & 1 ? v.w : v.z) : (w & 1 ? v.y : v.x);
+    return __uint_as_float(DT == kBF16 ? (j & 1 ? word & 0xffff0000u : word << 16) : word);
+}
+
 // The elements of a row at or above a bound, as they are found.
 template <int DT>
 struct Collector {
@@ -773,12 +857,17 @@ struct Collector {
         ElemTraits<DT>::unpack(raw, x);
         uint32_t hits = 0;
 #pragma unroll
-        for (int j = 0; j < EPV; ++j) hits += above(x[j]) ? 1u : 0u;
+        for (int j = 0; j < EPV; ++j) hits |= above(x[j]) ? 1u << j : 0u;
         if (hits == 0 || over()) return;
-        uint32_t pos = atomicAdd(&sh.n_cand, hits);
+        uint32_t pos = atomicAdd(&sh.n_cand, static_cast<uint32_t>(__popc(hits)));
+        if ((hits & (hits - 1)) == 0) {        // mostly one
+            const int j = __ffs(hits) - 1;
+            place(pick_element<DT>(raw, j), pos, vi * EPV + j - g.pre);
+        } else {
 #pragma unroll
-        for (int j = 0; j < EPV; ++j)
-            if (above(x[j])) place(x[j], pos++, vi * EPV + j - g.pre);
+            for (int j = 0; j < EPV; ++j)
+                if (hits >> j & 1u) place(x[j], pos++, vi * EPV + j - g.pre);
+        }
     }
     // A vector that sticks out of the row; each(x) is told its elements.
     template <class F>
@@ -965,11 +1054,13 @@ __device__ __forceinline__ void collect_mass(const RowGeom& g, const LaneSpan& s
     if ((threadIdx.x & 31) == 31) sh.warp_above[threadIdx.x >> 5] = m;
 }
 
-// log2 of the groups of threads per warp whose maxima bound a top-k of a cluster of S blocks: at least 3/2 k groups in the
-// cluster, if there are that many threads.
+// log2 of the groups of threads per warp whose maxima bound a top-k of a cluster of S blocks, if there are that many threads: in
+// the cluster at least 3/2 k groups, which leave about 1.65 k candidates; 4 k where that keeps the candidates within 128, of
+// which a warp sorts four per lane and not eight (draft step of 32 rows of 304 KB, top-k 100: 11.6 -> 9.3 us).
 inline int choose_groups(int S, int k) {
+    const long want = k > 64 && k <= 112 ? 4L * k : (3L * k + 1) / 2;
     int g = 0;
-    while (g < 5 && 2L * (kWarps * S << g) < 3L * k) ++g;
+    while (g < 5 && (kWarps * S << g) < want) ++g;
     return g;
 }
 
@@ -1000,7 +1091,8 @@ __device__ __forceinline__ void group_bound(SelectShared& sh, float best, int sh
     } else if (tid < 32) {
         uint32_t top;
         const uint32_t key = n <= 128 ? kth_bound<4>(sh.group_max, n, static_cast<uint32_t>(k), lane, top)
-                                      : kth_bound<kOneWarp / 32>(sh.group_max, n, static_cast<uint32_t>(k), lane, top);
+                             : n <= 256 ? kth_bound<8>(sh.group_max, n, static_cast<uint32_t>(k), lane, top)
+                                        : kth_bound<kOneWarp / 32>(sh.group_max, n, static_cast<uint32_t>(k), lane, top);
         if (lane == 0) {
             sh.bound_key = key;
             sh.tied = key == top;
@@ -1211,6 +1303,7 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
                     const uint2 o = ld_remote8(map_to_rank(smem_addr(&sh.cand[t]), r));
                     scratch->pool[first + t] = Candidate{o.x, o.y};
                 }
+                if (tid == 0 && total < kPoolCap) scratch->pool[total] = Candidate{0u, 0xffffffffu};
                 __syncthreads();
                 verdict = finish_pool<DT, kDraft, kTopK>(sh, *scratch, static_cast<int>(total), a, use_p, row_mass, row, tid,
                                                   key_out, tell);
