@@ -207,7 +207,14 @@ int pick_draft_cluster(const svip_ctx* ctx, long rows, int V, int dtype) {
 //            gain more (8 rows of 608 KB 11.2 us with 8, 10.8 with 6, flat 42.8 and 48.1; of 512 KB 11.1 and 11.7, flat 37.1
 //            and 43.2; of 1 MB 13.8 and 12.5, flat 54.6 and 62.4; 16 rows of 608 KB 13.9 and 12.1, flat 57.4 and 55.2)
 // and 2 rather than 1 as long as it fits (144 rows of 304 KB: 18.0 against 21.4 us).  Launches that fit with no size
-// are cut as those of the other kernels.
+// are cut as those of the other kernels; only the nucleus alone, whose second pass over the row is as long as the first, takes 3
+// where that is at most two full rounds of blocks (up to 6/5 rows per SM) or where the rows are so long (768 KB) that fewer blocks
+// per row would bring more rows than L2 holds between the two passes.  us with the number of the other kernels and with 3:
+//              159 rows      177 rows      198 rows (not)          240 rows      330 rows      600 rows
+//     250 KB   28.5 25.4     28.8 26.0     29.4 32.7      720 KB   54.2 57.0     72.3 73.2    118.1 119.5 (not)
+//     304 KB   30.4 27.6     28.2 28.2     29.2 34.9      800 KB   61.7 60.7     84.5 77.8    137.0 127.0
+//     512 KB   46.6 36.7     42.1 37.5     44.2 45.0      920 KB   68.4 66.8     95.0 85.7    158.9 141.7
+//     608 KB   37.2 34.9     39.1 35.9     42.6 45.9     1024 KB   75.7 70.6 (225 rows)  101.5 87.3 (300)  141.4 118.0 (450)
 int pick_threshold_cluster(const svip_ctx* ctx, long rows, int V, int dtype, bool top_k) {
     if (ctx->cluster_override > 0) return ctx->cluster_override;
     const long nvec = (static_cast<long>(V) * (dtype == SVIP_BF16 ? 2 : 4) + 15) / 16;
@@ -218,6 +225,8 @@ int pick_threshold_cluster(const svip_ctx* ctx, long rows, int V, int dtype, boo
         if (top_k ? S == 3 || (S == 6 && resident(4)) : (S == 8 && rows > 8) || (S == 3 && nvec * 16 < (256L << 10))) continue;
         return S;
     }
+    const long kb = nvec * 16 >> 10;
+    if (!top_k && (kb >= 768 || (kb >= 240 && 5 * rows <= 6L * ctx->num_sms))) return 3;
     return pick_cluster(ctx, rows, V, dtype);
 }
 
