@@ -145,7 +145,7 @@ __device__ __forceinline__ void stream_pair(const RowGeom& g, const RowGeom& gq,
         f(x, d);
     };
     int k = 0;
-    for (; k + 2 * kDepth <= span.full; k += kDepth) {      // steady state: every prefetch is in range
+    for (; k + 2 * kDepth <= n; k += kDepth) {      // steady state: every prefetch is in range
 #pragma unroll
         for (int s = 0; s < kDepth; ++s) step(s, true);
         pt += 32 * dir * kDepth;

@@ -606,12 +606,9 @@ __device__ __forceinline__ Partial warp_merge(Partial t, float c) {
 
 // What one lane of the warp reads of its segment: the vectors that lie inside the row go through the ring, vector
 // vi0 + 32 * it through slot it % kStages; the ones that stick out of the row (`head`, `tail`; set for lane 0 only)
-// are read apart.  Loops over whole rings are bounded by `full`, which is the same in all lanes: bounded by n, which differs by
-// one between them, the two parts of a warp went through different loops one after the other wherever n was about a multiple
-// of the ring.
+// are read apart.
 struct LaneSpan {
     int vi0, n;
-    int full;       // vectors that every lane of the warp has: n or n - 1
     bool head, tail;
     const uint4* src;
 };
@@ -630,7 +627,6 @@ __device__ __forceinline__ LaneSpan lane_span(const RowGeom& g, int seg, int lan
     s.tail = lane == 0 && tail_edge && v_hi == g.nvec && v_lo < v_hi && !(g.nvec == 1 && head_edge);
     s.vi0 = i_lo + lane;
     s.n = i_hi > s.vi0 ? (i_hi - s.vi0 + 31) >> 5 : 0;
-    s.full = max(i_hi - i_lo, 0) >> 5;
     s.src = g.base + s.vi0;
     return s;
 }
@@ -648,7 +644,7 @@ __device__ __forceinline__ void stream_interior(const LaneSpan& s, uint32_t slot
         cp_async_commit();
     }
     int it = 0;
-    for (; it + kStages <= s.full; it += kStages) {
+    for (; it + kStages <= s.n; it += kStages) {
 #pragma unroll
         for (int k = 0; k < kStages; ++k) {
             cp_async_wait<kStages - 1>();
@@ -660,7 +656,6 @@ __device__ __forceinline__ void stream_interior(const LaneSpan& s, uint32_t slot
         if (stop()) it = s.n;
     }
     cp_async_wait<0>();
-#pragma unroll 1
     for (; it < s.n; ++it) f(lds128(slot0 + (it & (kStages - 1)) * kSlotStride), s.vi0 + 32 * it);
 }
 
@@ -690,7 +685,7 @@ __device__ __forceinline__ Partial reduce_segment(const RowGeom& g, const LaneSp
     constexpr uint32_t kSlotStride = kThreads * 16;
     // vectors that stick out of the row are folded apart, by lane 0, with their outside masked
     const bool fold_head = span.head, fold_tail = span.tail;
-    const int vi0 = span.vi0, n = span.n, full = span.full;
+    const int vi0 = span.vi0, n = span.n;
     const uint4* src = span.src;
 #pragma unroll
     for (int s = 0; s < kStages; ++s) {
@@ -733,7 +728,7 @@ __device__ __forceinline__ Partial reduce_segment(const RowGeom& g, const LaneSp
         }
         int it = 0;
         // steady state: every prefetch is in range, slot numbers are compile-time constants
-        for (; it + 2 * kStages <= full; it += kStages) {
+        for (; it + 2 * kStages <= n; it += kStages) {
             const uint4* p = src + 32 * it;
 #pragma unroll
             for (int s = 0; s < kStages; ++s) {
@@ -749,7 +744,7 @@ __device__ __forceinline__ Partial reduce_segment(const RowGeom& g, const LaneSp
             acc_check<kMode>(t, c);
         }
         // last full ring: same static slots, prefetches only where the segment still has vectors
-        for (; it + kStages <= full; it += kStages) {
+        for (; it + kStages <= n; it += kStages) {
             const uint4* p = src + 32 * it;
 #pragma unroll
             for (int s = 0; s < kStages; ++s) {
@@ -764,19 +759,21 @@ __device__ __forceinline__ Partial reduce_segment(const RowGeom& g, const LaneSp
             }
             acc_check<kMode>(t, c);
         }
-        // at most kStages vectors left, all of them already in flight: `it` is a multiple of kStages, so vector it + k
-        // sits in slot k.  Unrolled like the loops above: small launches spend all their time here (RFIG).
+        // fewer than kStages vectors left, all of them already in flight: `it` is a multiple of
+        // kStages, so vector it + k sits in slot k.  Unrolled, because small launches spend their whole stream here (draft
+        // step of 16 rows of 200 KB bf16: rolled 6.0 us, unrolled 5.05; greedy round of 8 rows of 200 KB fp32, 5 steps and
+        // the verification, 23.4 and 22.2), with one test a vector (ring loops bounded by what all lanes of the warp have,
+        // and a second test per vector here: 32 rows of 304 KB 5.73 instead of 5.61, 32 such steps and a verification that
+        // stops at the first rejection 225 instead of 219).
         cp_async_wait<0>();
 #pragma unroll
-        for (int s = 0; s < kStages; ++s) {
-            if (it + s > full) break;
-            if (it + s < n) {
-                const uint4 raw = lds128(slot0 + s * kSlotStride);
-                float x[EPV];
-                ElemTraits<DT>::unpack(raw, x);
-                if (kThr) drop_below<EPV>(x, thr);
-                fold_fast<EPV, kMode, kIdx>(x, vi0 + 32 * (it + s), t);
-            }
+        for (int s = 0; s < kStages - 1; ++s) {
+            if (it + s >= n) break;
+            const uint4 raw = lds128(slot0 + s * kSlotStride);
+            float x[EPV];
+            ElemTraits<DT>::unpack(raw, x);
+            if (kThr) drop_below<EPV>(x, thr);
+            fold_fast<EPV, kMode, kIdx>(x, vi0 + 32 * (it + s), t);
         }
         acc_check<kMode>(t, c);
         if (fold_tail) {
