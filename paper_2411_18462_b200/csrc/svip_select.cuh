@@ -924,7 +924,8 @@ __device__ __forceinline__ float stream_maxima(const LaneSpan& s, uint32_t slot0
         left = st.rounds;
     };
     int it = 0;
-    for (; it + kStages <= s.n; it += kStages) {
+    const int full = fewest_vectors(s);
+    for (; it + kStages <= full; it += kStages) {
 #pragma unroll
         for (int k = 0; k < kStages; ++k) {
             cp_async_wait<kStages - 1>();
