@@ -126,7 +126,8 @@ struct SelectShared {
             uint32_t tot_cnt[256];            // the cluster's histogram
             unsigned long long tot_mass[256];
         };
-        uint32_t vec_list[kCandPerBlock];     // candidate path: stretches (top-k) or vectors with an element at or above the bound
+        uint32_t vec_list[kCandPerBlock];     // nucleus alone: vectors with an element at or above the bound
+        uint16_t stretch_list[kStretches * kThreads];   // top-k: stretches that may have one; room for every stretch of a block
     };
     float blk_max;                        // this block's largest logit
     unsigned long long blk_above;         // this block's mass of the elements >= tau_k
@@ -139,7 +140,7 @@ struct SelectShared {
     unsigned long long bar_group;         // all group maxima have landed
     unsigned long long bar_pool;          // block 0: headers and candidates of all blocks have landed
     unsigned long long bar_verdict;       // the verdict has landed
-    uint32_t n_vec;                       // how many of these there are (may exceed the capacity)
+    uint32_t n_vec;                       // how many of these there are (of vectors, may exceed the capacity)
     uint32_t n_cand;                      // how many candidates this block found (may exceed the capacity)
     uint32_t bound_key;                   // lower bound of the threshold
     uint32_t better[kMaxCluster];         // ... and a better one that each block finds, if they do not fit
@@ -817,7 +818,7 @@ struct MassSum {
     }
 };
 
-// Where a block collects its candidates, and lists the vectors that hold them.
+// Where a block collects its candidates, and (nucleus alone) lists the vectors that hold them.
 struct CollectInto {
     Candidate* cand;
     uint32_t cap;
@@ -973,40 +974,46 @@ __device__ __forceinline__ void collect_top(const RowGeom& g, const LaneSpan& s,
             }
         }
     } else {
+        // Only threads whose largest element reaches the bound list stretches, since half a key does not tell: of logits that are
+        // large against their spread, most stretches of a row agree with the bound in it (20 +- 0.01, 64 rows of 256000 fp32, top-k
+        // 50: 17.1 us; with every thread's stretches listed 35, with a list of 1024 that is taken to mean too many candidates 215).
         const uint32_t cut = c.lowest ? 0u : sh.bound_key >> 16;
         const int vectors = st.rounds * kStages;
-        for (int e = 0; e * vectors < s.n; ++e) {
-            if (sh.stretch_key[e][tid] < cut) continue;
-            const uint32_t pos = atomicAdd(&sh.n_vec, 1u);
-            if (pos < to.vec_cap) to.vec_list[pos] = static_cast<uint32_t>(e * kThreads + tid);
+        if (c.above(best)) {
+            for (int e = 0; e * vectors < s.n; ++e)
+                if (sh.stretch_key[e][tid] >= cut) sh.stretch_list[atomicAdd(&sh.n_vec, 1u)] = static_cast<uint16_t>(e * kThreads + tid);
         }
         __syncthreads();
-        const uint32_t n_hit = sh.n_vec;
-        // kStages threads per stretch, which take its vectors in turn; two vectors of a thread under way at a time.  Of a set
-        // that does not fit, a top-k still wants as many as there is room for (see better_bound).
-        const uint32_t items = min(n_hit, to.vec_cap) * kStages;
+        // kStages threads per stretch, which take its vectors in turn; of bf16 rows two vectors of a thread are under way at a time
+        // (of fp32 rows the registers for it have to be spilled: draft step of 256 rows of 1 MB 55.1 us, one at a time 52.0; bf16,
+        // 288 rows of 304 KB: 20.5, one at a time 21.0).  Of a set that does not fit, a top-k still wants as many as there is room for
+        // (see better_bound).
+        const uint32_t items = sh.n_vec * kStages;
+        const int inside = g.nvec - ((g.pre + g.V) % Collector<DT>::EPV != 0 ? 1 : 0);     // where a vector that sticks out begins
         for (int r = 0; r < st.rounds; ++r) {
-            const auto vector_of = [&](uint32_t i, LaneSpan& o) {      // which one of the lane's vectors, or -1
+            const auto vector_of = [&](uint32_t i) {      // which vector of the row, or -1
                 if (i >= items) return -1;
-                const uint32_t code = to.vec_list[i / kStages];
+                const uint32_t code = sh.stretch_list[i / kStages];
                 const int t = static_cast<int>(code % kThreads);
-                o = lane_span<DT>(g, rank * kWarps + (t >> 5), t & 31);
-                const int it = static_cast<int>(code / kThreads) * vectors + r * kStages + static_cast<int>(i % kStages);
-                return it < o.n ? it : -1;
+                int lo, hi;
+                seg_range(g, rank * kWarps + (t >> 5), lo, hi);
+                const int first = lo == 0 && g.pre > 0 ? 1 : lo;        // as lane_span() has it
+                const int vi = first + (t & 31) + 32 * (static_cast<int>(code / kThreads) * vectors + r * kStages + static_cast<int>(i % kStages));
+                return vi < min(hi, inside) ? vi : -1;
             };
-            for (uint32_t i = tid; i < items && !c.over(); i += 2 * kThreads) {
-                LaneSpan o0, o1;
-                const int it0 = vector_of(i, o0), it1 = vector_of(i + kThreads, o1);
-                uint4 raw0 = make_uint4(0, 0, 0, 0), raw1 = raw0;
-                if (it0 >= 0) raw0 = ld_vec(o0.src + 32 * it0);
-                if (it1 >= 0) raw1 = ld_vec(o1.src + 32 * it1);
-                if (it0 >= 0) c.visit(raw0, o0.vi0 + 32 * it0);
-                if (it1 >= 0) c.visit(raw1, o1.vi0 + 32 * it1);
+            constexpr int kAtOnce = DT == kBF16 ? 2 : 1;
+            for (uint32_t i = tid; i < items && !c.over(); i += kAtOnce * kThreads) {
+                int vi[kAtOnce];
+                uint4 raw[kAtOnce];
+#pragma unroll
+                for (int q = 0; q < kAtOnce; ++q) {
+                    vi[q] = vector_of(i + q * kThreads);
+                    raw[q] = vi[q] >= 0 ? ld_vec(g.base + vi[q]) : make_uint4(0, 0, 0, 0);
+                }
+#pragma unroll
+                for (int q = 0; q < kAtOnce; ++q)
+                    if (vi[q] >= 0) c.visit(raw[q], vi[q]);
             }
-        }
-        if (n_hit > to.vec_cap) {
-            __syncthreads();
-            if (tid == 0) atomicAdd(&sh.n_cand, to.cap + 1);
         }
     }
     if (s.head) c.edge(0, [](float) {});
@@ -1306,7 +1313,7 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
                 }
                 if (tid == 0 && total < kPoolCap) scratch->pool[total] = Candidate{0u, 0xffffffffu};
                 __syncthreads();
-                verdict = finish_pool<DT, kDraft, kTopK>(sh, *scratch, static_cast<int>(total), a, use_p, row_mass, row, tid,
+                return finish_pool<DT, kDraft, kTopK>(sh, *scratch, static_cast<int>(total), a, use_p, row_mass, row, tid,
                                                   key_out, tell);
             }
         }
@@ -1357,7 +1364,7 @@ __global__ void __launch_bounds__(kThreads, 2) row_threshold_kernel(ThresholdArg
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const char* rp = static_cast<const char*>(a.logits) +
                      static_cast<size_t>(row) * a.row_stride * ElemTraits<DT>::kBytes;
-    const RowGeom g = make_geom<DT>(rp, a.V, S * kWarps);
+    RowGeom g = make_geom<DT>(rp, a.V, S * kWarps);
     const uint32_t slot0 = static_cast<uint32_t>(__cvta_generic_to_shared(ring)) + tid * 16;
     const bool use_p = a.top_p < 1.0f;
     // a small k against the number of threads of the cluster, or the nucleus alone: two passes over the row
@@ -1387,6 +1394,14 @@ __global__ void __launch_bounds__(kThreads, 2) row_threshold_kernel(ThresholdArg
             draft_at_threshold<DT>(a, S, rank, row, tid, g, slot0, key_t ? key_value(key_t) : neg_inf());
             return;
         }
+    }
+
+    if (!kDraft) {
+        // The geometry once more: kept across the candidate path it costs registers there, and few rows come here (threshold of 288
+        // rows of 304 KB, top-k 50: 20.5 us, this way 19.3; the draft step does not gain).
+        int again = row;
+        asm volatile("" : "+r"(again));
+        g = make_geom<DT>(static_cast<const char*>(a.logits) + static_cast<size_t>(again) * a.row_stride * ElemTraits<DT>::kBytes, a.V, S * kWarps);
     }
 
     if (kTopK) {
