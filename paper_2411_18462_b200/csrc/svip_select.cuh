@@ -26,7 +26,7 @@ constexpr int kHistCopies = 8;           // interleaved copies of the histogram:
                                          // lanes that meet in one bin mostly hit different words and banks
 constexpr float kMassScale = 1099511627776.0f;   // 2^40
 constexpr int kPoolCap = 2048;           // candidates of the whole cluster
-constexpr int kCandPerBlock = 1024;      // candidates one of several blocks may collect
+constexpr int kCandPerBlock = 1024;      // top-k: candidates one of several blocks may collect (nucleus alone: kPoolCap)
 constexpr int kSorted = 256;             // up to this many candidates are put in order, the keys by one warp
 constexpr int kMaxGroups = 2048;         // groups of threads whose maxima give the bound of a top-k
 constexpr int kOneWarp = 512;            // up to this many group maxima are searched by one warp
@@ -112,12 +112,17 @@ struct SelectShared {
         struct {
             Candidate landing[kPoolCap];      // candidate path, block 0: the peers' candidates, one region per block (the
                                               // candidates of a block alone)
-            uint16_t stretch_key[kStretches][kThreads];   // top-k, rows that do not fit the ring: see stream_maxima
+            union {
+                struct {                      // top-k
+                    uint16_t stretch_key[kStretches][kThreads];   // rows that do not fit the ring: see stream_maxima
+                    union {
+                        alignas(16) float group_max[kMaxGroups];  // group maxima of the whole cluster
+                        Candidate cand[kCandPerBlock];            // then this block's elements at or above the bound
+                    };
+                };
+                Candidate cand_alone[kPoolCap];   // nucleus alone: likewise
+            };
         };
-    };
-    union {
-        alignas(16) float group_max[kMaxGroups];   // candidate path: group maxima of the whole cluster
-        Candidate cand[kCandPerBlock];        // then this block's elements at or above the bound
     };
     union {
         struct {
@@ -126,7 +131,7 @@ struct SelectShared {
             uint32_t tot_cnt[256];            // the cluster's histogram
             unsigned long long tot_mass[256];
         };
-        uint32_t vec_list[kCandPerBlock];     // nucleus alone: vectors with an element at or above the bound
+        uint32_t vec_list[kPoolCap];          // nucleus alone: vectors with an element at or above the bound
         uint16_t stretch_list[kStretches * kThreads];   // top-k: stretches that may have one; room for every stretch of a block
     };
     float blk_max;                        // this block's largest logit
@@ -818,12 +823,10 @@ struct MassSum {
     }
 };
 
-// Where a block collects its candidates, and (nucleus alone) lists the vectors that hold them.
+// Where a block collects its candidates.
 struct CollectInto {
     Candidate* cand;
     uint32_t cap;
-    uint32_t* vec_list;
-    uint32_t vec_cap;
 };
 
 // Element j of a vector.
@@ -1040,17 +1043,17 @@ __device__ __forceinline__ void collect_mass(const RowGeom& g, const LaneSpan& s
     } else {
         // the streaming loop only lists the vectors, which are few, and all threads look at them afterwards: with the
         // elements looked at inside the unrolled loop, 2304 rows of 304 KB took 272 us instead of 174
-        auto full = [&]() { return *static_cast<volatile uint32_t*>(&sh.n_vec) > to.vec_cap; };
+        auto full = [&]() { return *static_cast<volatile uint32_t*>(&sh.n_vec) > kPoolCap; };
         stream_interior(s, slot0, [&](const uint4& raw, int vi) {
             if (has(raw) && !full()) {
                 const uint32_t pos = atomicAdd(&sh.n_vec, 1u);
-                if (pos < to.vec_cap) to.vec_list[pos] = static_cast<uint32_t>(vi);
+                if (pos < kPoolCap) sh.vec_list[pos] = static_cast<uint32_t>(vi);
             }
         }, full);
         __syncthreads();
         const uint32_t nv = sh.n_vec;
-        if (nv <= to.vec_cap) {
-            for (uint32_t i = threadIdx.x; i < nv; i += kThreads) c.visit(ld_vec(g.base + to.vec_list[i]), to.vec_list[i]);
+        if (nv <= kPoolCap) {
+            for (uint32_t i = threadIdx.x; i < nv; i += kThreads) c.visit(ld_vec(g.base + sh.vec_list[i]), sh.vec_list[i]);
         } else {
             __syncthreads();
             if (threadIdx.x == 0) atomicAdd(&sh.n_cand, to.cap + 1);
@@ -1194,8 +1197,8 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
     // A block alone collects where the peers' candidates would land.  Otherwise every block collects at home; its first
     // kPoolCap / S candidates are pushed to block 0, which has that much room for each, and fetches the others of a block in
     // whose part of the row the likely tokens are gathered.
-    const CollectInto to = S == 1 ? CollectInto{sh.landing, kPoolCap, reinterpret_cast<uint32_t*>(sh.cand), 2 * kCandPerBlock}
-                                  : CollectInto{sh.cand, kCandPerBlock, sh.vec_list, kCandPerBlock};
+    Candidate* const home = kTopK ? sh.cand : sh.cand_alone;
+    const CollectInto to = S == 1 ? CollectInto{sh.landing, kPoolCap} : CollectInto{home, kTopK ? kCandPerBlock : kPoolCap};
     const uint32_t region = kPoolCap / S;
     const bool resident = g.vps <= 32 * kStages;
     const Stretches stretches(g);
@@ -1264,7 +1267,7 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
             const uint32_t sent = mine <= to.cap ? min(mine, region) : 0u;
             const uint32_t bar0 = map_to_rank(smem_addr(&sh.bar_pool), 0);
             for (uint32_t i = tid; i < sent; i += kThreads)
-                push8(map_to_rank(smem_addr(&sh.landing[rank * region + i]), 0), bar0, sh.cand[i].key, sh.cand[i].idx);
+                push8(map_to_rank(smem_addr(&sh.landing[rank * region + i]), 0), bar0, home[i].key, home[i].idx);
             if (tid == 0) {
                 push16(map_to_rank(smem_addr(&sh.header[rank]), 0), bar0, mine, static_cast<uint32_t>(my_mass),
                        static_cast<uint32_t>(my_mass >> 32), 0u);
@@ -1308,7 +1311,7 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
                 for (uint32_t t = (warp / kMaxCluster) * 32 + lane; t < here; t += 64) scratch->pool[first + t] = from[t];
                 // the block stays, and keeps its candidates, until it hears the verdict
                 for (uint32_t t = here + (warp / kMaxCluster) * 32 + lane; t < nr; t += 64) {
-                    const uint2 o = ld_remote8(map_to_rank(smem_addr(&sh.cand[t]), r));
+                    const uint2 o = ld_remote8(map_to_rank(smem_addr(&home[t]), r));
                     scratch->pool[first + t] = Candidate{o.x, o.y};
                 }
                 if (tid == 0 && total < kPoolCap) scratch->pool[total] = Candidate{0u, 0xffffffffu};
