@@ -207,14 +207,20 @@ int pick_draft_cluster(const svip_ctx* ctx, long rows, int V, int dtype) {
 //            gain more (8 rows of 608 KB 11.2 us with 8, 10.8 with 6, flat 42.8 and 48.1; of 512 KB 11.1 and 11.7, flat 37.1
 //            and 43.2; of 1 MB 13.8 and 12.5, flat 54.6 and 62.4; 16 rows of 608 KB 13.9 and 12.1, flat 57.4 and 55.2)
 // and 2 rather than 1 as long as it fits (144 rows of 304 KB: 18.0 against 21.4 us).  Launches that fit with no size
-// are cut as those of the other kernels; only the nucleus alone, whose second pass over the row is as long as the first, takes 3
-// where that is at most two full rounds of blocks (up to 6/5 rows per SM) or where the rows are so long (768 KB) that fewer blocks
-// per row would bring more rows than L2 holds between the two passes.  us with the number of the other kernels and with 3:
-//              159 rows      177 rows      198 rows (not)          240 rows      330 rows      600 rows
-//     250 KB   28.5 25.4     28.8 26.0     29.4 32.7      720 KB   54.2 57.0     72.3 73.2    118.1 119.5 (not)
-//     304 KB   30.4 27.6     28.2 28.2     29.2 34.9      800 KB   61.7 60.7     84.5 77.8    137.0 127.0
-//     512 KB   46.6 36.7     42.1 37.5     44.2 45.0      920 KB   68.4 66.8     95.0 85.7    158.9 141.7
-//     608 KB   37.2 34.9     39.1 35.9     42.6 45.9     1024 KB   75.7 70.6 (225 rows)  101.5 87.3 (300)  141.4 118.0 (450)
+// are cut as those of the other kernels, but the nucleus alone, whose second pass over the row is as long as the first, takes 3
+// where that is at most two full rounds of blocks (rows of 384 KB up to 6/5 rows per SM, of 768 KB up to 4/3), and again from two
+// rows per SM on where the rows are so long (896 KB) that fewer blocks per row would bring more rows than L2 holds between the two
+// passes; between these flat rows lose more than the others gain.  us with the number of the other kernels and with 3, for rows
+// with a few likely tokens and for flat rows, which take the descent:
+//                               likely        flat                                       likely        flat
+//     160 x 250 KB fp32 (not)  20.3  21.9   117  116          180 x 1000 KB fp32        68.9  53.8   345  324
+//     160 x 297 KB bf16 (not)  28.1  28.0   159  140          200 x 1000 KB fp32 (not)  74.4  67.7   348  392
+//     160 x 390 KB bf16        34.5  32.6   201  172          200 x 1000 KB bf16 (not)  70.7  74.9   417  466
+//     177 x 390 KB bf16        35.0  33.1   201  173          280 x 1000 KB fp32 (not)  89.6  83.6   427  515
+//     160 x 500 KB fp32        32.4  31.5   209  181          300 x 1000 KB fp32       103.0  88.1   538  536
+//     160 x 703 KB fp32        44.9  40.5   252  238          300 x 1000 KB bf16       106.4  96.2   642  626
+//     280 x 781 KB fp32 (not)  68.8  70.1   343  424          600 x 1000 KB fp32       182.6 153.4   929  999
+//     280 x 781 KB bf16 (not)  71.9  77.9   404  494          600 x  781 KB fp32 (not) 137.1 128.4   745  817
 int pick_threshold_cluster(const svip_ctx* ctx, long rows, int V, int dtype, bool top_k) {
     if (ctx->cluster_override > 0) return ctx->cluster_override;
     const long nvec = (static_cast<long>(V) * (dtype == SVIP_BF16 ? 2 : 4) + 15) / 16;
@@ -226,7 +232,10 @@ int pick_threshold_cluster(const svip_ctx* ctx, long rows, int V, int dtype, boo
         return S;
     }
     const long kb = nvec * 16 >> 10;
-    if (!top_k && (kb >= 768 || (kb >= 240 && 5 * rows <= 6L * ctx->num_sms))) return 3;
+    if (!top_k) {
+        if (3 * rows <= 4L * ctx->num_sms && kb >= (5 * rows <= 6L * ctx->num_sms ? 384 : 768)) return 3;
+        if (rows >= 2L * ctx->num_sms && kb >= 896) return 3;
+    }
     return pick_cluster(ctx, rows, V, dtype);
 }
 

@@ -202,3 +202,18 @@ def test_flat_rows_leave_the_candidates_soon(ctx):
         x = -1.1 * np.log(np.arange(1, V + 1))
         rows = W.to_bf16_bits(np.stack([x[rng.permutation(V)] for _ in range(B)]).astype(np.float32))
         assert us_per_call(ctx, rows, 0, 0.95) < 1.02 * us_per_call(ctx, rows, V - 1, 0.95), (B, V)
+
+
+def test_flat_rows_are_cut_no_worse_than_by_the_other_kernels(ctx):
+    # long rows between 4/3 and 2 per SM.  Measured 1.0 to 1.06 times the best of one and two blocks per row; with three 1.3
+    rng = np.random.default_rng(8)
+    rows = rng.standard_normal((280, 200000), dtype=np.float32)
+    chosen = us_per_call(ctx, rows, 0, 0.95, calls=4)
+    best = []
+    try:
+        for S in (1, 2):
+            ctx.set_cluster_size(S)
+            best.append(us_per_call(ctx, rows, 0, 0.95, calls=4))
+    finally:
+        ctx.set_cluster_size(0)
+    assert chosen < 1.15 * min(best), (chosen, best)
