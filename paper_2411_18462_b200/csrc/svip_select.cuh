@@ -30,6 +30,7 @@ constexpr int kCandPerBlock = 1024;      // top-k: candidates one of several blo
 constexpr int kSorted = 256;             // up to this many candidates are put in order, the keys by one warp
 constexpr int kMaxGroups = 2048;         // groups of threads whose maxima give the bound of a top-k
 constexpr int kOneWarp = 512;            // up to this many group maxima are searched by one warp
+constexpr int kRetryTopK = 128;          // up to this k a second bound is tried where the candidates do not fit
 constexpr int kStretches = 8;            // maxima that a thread keeps of the vectors it streams
 
 struct ThresholdArgs {
@@ -1115,11 +1116,15 @@ __device__ __forceinline__ void group_bound(SelectShared& sh, float best, int sh
 // A better bound for a top-k whose candidates do not fit; the same in every block.  The maxima of large groups bound next to
 // nothing where the likely tokens are gathered in few warps (a vocabulary in order of frequency).  There every block that found
 // too many elements takes the maxima of its threads, or of their stretches of vectors, as groups, stores what reaches
-// the k-th largest of these (at least the first of them), and any block with k elements stored takes their k-th largest: a
+// the k-th largest of these (at least the first of them; a block alone whose row is in the ring goes by what it has stored, the 2048
+// that came first), and any block with k elements stored takes their k-th largest: a
 // bound for the row as well, and the blocks agree on the largest of these.  Rows of 50021 fp32 logits in order of frequency,
 // top-k 50, against the maxima of the smallest groups of the cluster (few rows) or the k-th largest of what happened to be
 // stored: 1 row 15.7 -> 13.3 us, 64 rows 22.4 -> 19.0, 300 rows 42.1 -> 36.6, 300 rows in reversed order 99.6 -> 35.9 (with
-// the descent in place of the second attempt 123).  A function of its own, because its code in line cost every top-k 3 %.
+// the descent in place of the second attempt 123).  A block alone with its row in the ring, 600 rows of 32000 bf16: top-k 50 30.8 us,
+// by the maxima of its threads first 49; top-k 100 39.5 and 90.  From a k of about 300 on those maxima say too little, and the attempt
+// comes before the descent and not in its place (64 rows of 32000 bf16, top-k 300, 18.8 us without and 26.4 with it), hence the line
+// at kRetryTopK, up to which it was seen to succeed.  A function of its own, because its code in line cost every top-k 3 %.
 template <int DT>
 __device__ __noinline__ uint32_t better_bound(SelectShared& sh, const CollectInto to, const RowGeom g, bool resident, uint32_t slot0,
                                               float best, int S, int rank, int k, unsigned* status) {
@@ -1127,7 +1132,7 @@ __device__ __noinline__ uint32_t better_bound(SelectShared& sh, const CollectInt
     const uint32_t want = static_cast<uint32_t>(k);
     const uint32_t found = sh.n_cand;
     uint32_t bound = 0, stored = min(found, to.cap);
-    if (found > to.cap) {
+    if (found > to.cap && (S > 1 || !resident)) {
         const Stretches st(g);
         const int groups = resident ? kThreads : st.count * kThreads;
         if (resident) {
@@ -1300,7 +1305,7 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
             const uint32_t total = __shfl_sync(0xffffffffu, end, kMaxCluster - 1);
             const bool fits = !__any_sync(0xffffffffu, count > to.cap) && total <= kPoolCap;
             if (!fits || total < static_cast<uint32_t>(kTopK ? a.top_k : 1)) {
-                verdict = kTopK && !fits && parity == 0 && !sh.tied ? kVerdictRetry : kVerdictDescend;
+                verdict = kTopK && !fits && parity == 0 && !sh.tied && a.top_k <= kRetryTopK ? kVerdictRetry : kVerdictDescend;
                 tell(verdict, 0u);
             } else {
                 // two warps copy the candidates of each block

@@ -177,6 +177,39 @@ def test_order_of_frequency_costs_little_more(ctx):
         assert us_per_call(ctx, x, 50, 1.0) < 2.7 * shuffled, B
 
 
+@pytest.mark.parametrize("S", [1, 2, 8])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_order_of_frequency_in_the_ring(ctx, oracle, S, bf16):
+    # rows that stay in the ring, with one block per row too; k on either side of where a second bound is tried
+    rng = np.random.default_rng(30 + S)
+    V = 16384 if not bf16 else 30011
+    x = -1.1 * np.log(np.arange(1, V + 1)) + 0.2 * rng.standard_normal((3, V))
+    x[1] = x[1][::-1]
+    rows = W.to_bf16_bits(x.astype(np.float32)) if bf16 else x.astype(np.float32)
+    u = rng.random(3).astype(np.float32)
+    ctx.set_cluster_size(S)
+    try:
+        for k in (20, 50, 100, 128, 129, 300, 1000):
+            if k <= S * 128:
+                check_truncated(ctx, oracle, rows, 0.8, k, 0.95, u, "S=%d k=%d" % (S, k))
+        assert ctx.read_status() == 0
+    finally:
+        ctx.set_cluster_size(0)
+
+
+def test_order_of_frequency_does_not_pay_for_attempts_that_fail(ctx):
+    # one block per row, in the ring: measured 1.5 times the shuffled vocabulary; with a bound from the threads' maxima first, which
+    # here is no better than the first one, 3.6
+    rng = np.random.default_rng(9)
+    V = 32000
+    x = (-1.1 * np.log(np.arange(1, V + 1)) + 0.2 * rng.standard_normal((600, V))).astype(np.float32)
+    shuffled = us_per_call(ctx, W.to_bf16_bits(np.ascontiguousarray(x[:, rng.permutation(V)])), 100, 0.9)
+    assert us_per_call(ctx, W.to_bf16_bits(x), 100, 0.9) < 2.2 * shuffled
+    # a large k: measured 1.45 times one so large that the row goes to the descent at once; with a second bound tried first 2.05
+    rows = W.to_bf16_bits(x[:64])
+    assert us_per_call(ctx, rows, 300, 1.0) < 1.75 * us_per_call(ctx, rows, 1000, 1.0)
+
+
 def test_gathered_sets_cost_what_spread_ones_do(ctx):
     # measured: 1.1 to 1.2 times; where the candidates of a block did not fit the table and the row took the descent 1.5 to 1.6
     rng = np.random.default_rng(2)
