@@ -507,26 +507,13 @@ __device__ __forceinline__ unsigned long long nucleus_target(float top_p, unsign
     return want > total ? total : want;
 }
 
-// Sums over the lanes of a warp of integers below 2^48 in magnitude: 24 bits and the rest are summed apart, in 32 bits each, which
-// takes no carries and half the instructions.
+// Sum over the lanes of a warp, modulo 2^64: 24, 24 and 16 bits apart, in 32 bits each.  All 64 bits: the weight of a row's
+// largest logit is 2 to the rounding error of max * c, which is not near 1 where |max| / T is above some 10^8.
 __device__ __forceinline__ unsigned long long warp_total_mass(unsigned long long v) {
     const uint32_t lo = __reduce_add_sync(0xffffffffu, static_cast<uint32_t>(v) & 0xffffffu);
-    const uint32_t hi = __reduce_add_sync(0xffffffffu, static_cast<uint32_t>(v >> 24));
-    return (static_cast<unsigned long long>(hi) << 24) + lo;
-}
-__device__ __forceinline__ long long warp_total_signed(long long v) {
-    const uint32_t lo = __reduce_add_sync(0xffffffffu, static_cast<uint32_t>(v) & 0xffffffu);
-    const int hi = __reduce_add_sync(0xffffffffu, static_cast<int>(v >> 24));
-    return static_cast<long long>(hi) * (1 << 24) + lo;
-}
-__device__ __forceinline__ unsigned long long warp_prefix_mass(unsigned long long v, int lane) {     // inclusive
-    uint32_t lo = static_cast<uint32_t>(v) & 0xffffffu, hi = static_cast<uint32_t>(v >> 24);
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t l = __shfl_up_sync(0xffffffffu, lo, o), h = __shfl_up_sync(0xffffffffu, hi, o);
-        if (lane >= o) { lo += l; hi += h; }
-    }
-    return (static_cast<unsigned long long>(hi) << 24) + lo;
+    const uint32_t mid = __reduce_add_sync(0xffffffffu, static_cast<uint32_t>(v >> 24) & 0xffffffu);
+    const uint32_t hi = __reduce_add_sync(0xffffffffu, static_cast<uint32_t>(v >> 48));
+    return (static_cast<unsigned long long>(hi) << 48) + (static_cast<unsigned long long>(mid) << 24) + lo;
 }
 
 // A block barrier that the warps may reach in different places of the code.
@@ -589,7 +576,7 @@ __device__ __forceinline__ void finish_by_key(PoolScratch& ps, int n, const Thre
             if (kTopK && key[j] >= key_t) kept += m;
         }
         const unsigned long long zk = kTopK ? warp_total_mass(kept) : row_mass;     // kTopK: of the candidates >= tau_k
-        const unsigned long long incl = warp_prefix_mass(sum, lane);
+        const unsigned long long incl = warp_scan_mass(sum, lane);
         if (zk > 0) {
             const unsigned long long want = nucleus_target(a.top_p, zk);
             unsigned long long cum = incl - sum;
@@ -625,7 +612,7 @@ __device__ __forceinline__ void finish_by_key(PoolScratch& ps, int n, const Thre
     const unsigned long long zt = warp_total_mass(z);
     if (lane == 0 && a.stats) a.stats[row] = kept_stats(row_max, zt, finite);
     if (!kDraft) return;
-    const long long aq = warp_total_signed(term);
+    const long long aq = static_cast<long long>(warp_total_mass(static_cast<unsigned long long>(term)));
     if (lane == 0) {
         const float Z = static_cast<float>(static_cast<double>(zt) / 1099511627776.0);
         const float A = static_cast<float>(static_cast<double>(aq) / 1099511627776.0);
@@ -648,7 +635,7 @@ __device__ __forceinline__ void sample_by_index(const PoolScratch& ps, int n, ui
         if (k < mine && ps.by_idx[lo + k].key >= key_t) sum += ps.mass_idx[lo + k];
         cum[k] = sum;
     }
-    const unsigned long long incl = warp_prefix_mass(sum, lane), before = incl - sum;
+    const unsigned long long incl = warp_scan_mass(sum, lane), before = incl - sum;
     const unsigned long long target = static_cast<unsigned long long>(static_cast<double>(u) * static_cast<double>(shfl_u64(incl, 31)));
     if (before <= target && target < incl) {      // exactly one lane: the target is less than the total
         int at = lo;

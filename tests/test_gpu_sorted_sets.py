@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 from paper_2411_18462_b200 import workloads as W
-from test_gpu_candidate_sets import check_truncated
+from test_gpu_candidate_sets import check_truncated, truncated
 
 pytestmark = pytest.mark.gpu
 
@@ -36,6 +36,46 @@ def test_sizes_of_sorted_sets(ctx, oracle, S, bf16):
                 check_truncated(ctx, oracle, rows, 1.0, 0, p, u, "nucleus S=%d n=%d p=%g" % (S, n, p))
             if n <= 128:
                 check_truncated(ctx, oracle, rows, 1.0, n, 0.9, u, "top-k S=%d n=%d" % (S, n))
+        assert ctx.read_status() == 0
+    finally:
+        ctx.set_cluster_size(0)
+
+
+def far_from_zero(bf16):
+    """A logit whose product with log2(e) is rounded by nearly 16, half a unit in the last place, and that error."""
+    c = np.float64(np.float32(1.4426950408889634))
+    x = np.arange(1.9e8, 3.7e8, 1e6 if bf16 else 1e3).astype(np.float32)
+    if bf16:
+        x = np.unique(W.bf16_bits_to_f32(W.to_bf16_bits(x)))
+    exact = x.astype(np.float64) * c                       # 48 bits: exact
+    error = exact - exact.astype(np.float32).astype(np.float64)
+    best = int(np.argmax(error))
+    return x[best], error[best]
+
+
+@pytest.mark.parametrize("S", [1, 4])
+@pytest.mark.parametrize("bf16", [False, True])
+def test_logits_far_from_zero(ctx, S, bf16):
+    # the mass of the largest logit is 2^40 times 2 to the rounding error of its product with log2(e): four of them make about 2^58
+    x, error = far_from_zero(bf16)
+    assert error > 14.5
+    V, n = 3001, 4
+    at = np.array([5, 700, 1501, 2999])
+    v = np.full((8, V), x - np.float32(6.4e7), dtype=np.float32)
+    v[:, at] = x
+    rows = W.to_bf16_bits(v) if bf16 else v
+    u = ((np.arange(8) + 0.5) / 8).astype(np.float32)
+    ctx.set_cluster_size(S)
+    try:
+        for k, p in ((4, 1.0), (4, 0.9), (0, 0.9)):
+            thr, stats, (tok, ent, _, _) = truncated(ctx, rows, 1.0, k, p, u)
+            label = "S=%d k=%d p=%g" % (S, k, p)
+            assert np.all(thr == x), label
+            assert np.array_equal(tok, at[np.floor(u * n).astype(int)]), (label, tok)
+            # ln 4 from terms of the size of the error in log2 units, each of 2-ulp exponentials
+            assert np.all(np.abs(ent - np.log(n)) <= 1e-4), (label, ent)
+            for st in stats:
+                assert np.all(st[:, 0] == x) and np.all(np.abs(st[:, 1] / (n * 2.0 ** error) - 1.0) <= 1e-5), (label, st)
         assert ctx.read_status() == 0
     finally:
         ctx.set_cluster_size(0)
