@@ -3,8 +3,10 @@ keys across the cut, rows without finite mass.  Oracle and tolerances are those 
 import numpy as np
 import pytest
 
+import svip_testlib as tl
 from paper_2411_18462_b200 import workloads as W
 from test_gpu_candidate_sets import check_truncated, truncated
+from test_gpu_truncation import check
 
 pytestmark = pytest.mark.gpu
 
@@ -77,5 +79,44 @@ def test_logits_far_from_zero(ctx, S, bf16):
             for st in stats:
                 assert np.all(st[:, 0] == x) and np.all(np.abs(st[:, 1] / (n * 2.0 ** error) - 1.0) <= 1e-5), (label, st)
         assert ctx.read_status() == 0
+    finally:
+        ctx.set_cluster_size(0)
+
+
+@pytest.mark.parametrize("S", [1, 4])
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("V", [200, 20011])
+def test_rows_without_finite_mass(ctx, oracle, V, bf16, S):
+    # their draft step is streamed at the threshold by the whole cluster, after block 0 has sorted the candidates: the same results as
+    # from the two separate calls, next to rows that are finished from their candidates.  With the short rows every token is a candidate
+    import torch
+    rng = np.random.default_rng(V + S)
+    x = (rng.standard_normal((7, V)) * 2.0).astype(np.float32)
+    x[1] = -np.inf
+    x[2, V // 3] = np.inf
+    x[3, V // 2] = 2.0e29                 # beyond what counts as finite
+    x[4] = np.nan
+    x[5] = -2.0e29
+    finite = [0, 6]
+    rows = W.to_bf16_bits(x) if bf16 else x
+    u = rng.random(7).astype(np.float32)
+    d, dt = tl.to_device(rows), tl.dtype_code(rows)
+    ctx.set_cluster_size(S)
+    try:
+        for k, p in ((50, 1.0), (50, 0.9), (1, 1.0), (0, 0.9)):
+            label = "V=%d S=%d k=%d p=%g" % (V, S, k, p)
+            ctx.read_status()
+            thr, stats, step = truncated(ctx, rows, 1.0, k, p, u)
+            assert ctx.read_status() == 1, label        # a row without finite mass, and nothing else
+            z = lambda *s, d=torch.float32: torch.zeros(*s, dtype=d, device="cuda")  # noqa: E731
+            st, tok, ent, stop = z(7, 2), z(7, d=torch.int32), z(7), z(7, d=torch.uint8)
+            ctx.draft_step_filtered(d, dt, 7, V, V, 1.0, 0.3, tl.to_device(u), None, tl.to_device(thr), tok, ent, stop, st)
+            torch.cuda.synchronize()
+            other = [b for b in range(7) if b not in finite]
+            for got, want in zip((step[0], step[1], step[2], stats[0]), (tok, ent, stop, st)):
+                assert np.array_equal(got[other], want.cpu().numpy()[other], equal_nan=got.dtype == np.float32), label
+            check(oracle, rows[finite], 1.0, k, p, thr[finite], label)
+            tl.check_draft_against_oracle(oracle, oracle.mask_below(rows[finite], thr[finite].astype(np.float64)), 1.0, 0.3, u[finite],
+                                          tuple(a[finite] for a in step[:3]) + (None,), label)
     finally:
         ctx.set_cluster_size(0)
