@@ -1,7 +1,6 @@
-"""The candidate path of the threshold kernel where it changes form: sets of candidates around what is sorted (512) and
+"""The candidate path of the threshold kernel where it changes form: sets of candidates around what was once sorted (512) and
 what is held at all (2048), spread over the row or gathered in one block's part of it, segments that stay in the
-shared-memory ring and segments that do not, ties at the bound, and a bound from half of the row that lets too many
-candidates in.  Oracle and tolerances are those of test_gpu_truncation."""
+shared-memory ring and segments that do not, ties at the bound, and a first bound that lets too many candidates in.  Oracle and tolerances are those of test_gpu_truncation."""
 import numpy as np
 import pytest
 
@@ -81,26 +80,37 @@ def test_ties_at_the_top_k_bound(ctx, oracle, S, V, n):
         ctx.set_cluster_size(0)
 
 
-def test_bound_from_half_of_the_row_lets_too_many_in(ctx, oracle):
-    # more than 48 MB of logits: the bound comes from the first half of every segment, where this row has nothing
-    V, n = 152064, 100
+def group_maxima(row, S, per_warp):
+    """Maxima of the groups of neighbouring threads from which the first bound of a top-k is taken: the vectors of a warp's segment
+    go to its lanes in turn.  fp32 rows that start and end at a vector."""
+    vectors = row.reshape(-1, 4).max(axis=1)
+    nseg = 16 * S
+    vps = ((vectors.size + nseg - 1) // nseg + 7) // 8 * 8
+    out = []
+    for lo in range(0, vectors.size, vps):
+        seg = vectors[lo:lo + vps]
+        group = np.arange(seg.size) % 32 * per_warp // 32
+        out += [seg[group == j].max() for j in range(per_warp)]
+    return np.array(out)
+
+
+def test_likely_tokens_in_few_groups_of_threads(ctx, oracle):
+    # rows that do not fit the ring, their likely tokens all in one warp's segment: most of the group maxima are those of unlikely
+    # tokens, the first bound lets in more than the tables hold, and the maxima of stretches have to give a second one
+    V, n, k = 152064, 100, 50
     rng = np.random.default_rng(5)
     x = rng.standard_normal((n, V)).astype(np.float32)
-    x[::7] -= 20.0
-    for S in (1, 2):
+    for S, per_warp in ((1, 8), (2, 4)):       # as many groups as have at least 3/2 k
         rows = x.copy()
-        nseg = 16 * S
-        vps = ((V // 4 + nseg - 1) // nseg + 7) // 8 * 8
-        first = np.zeros(V, dtype=bool)
-        for seg in range(nseg):
-            lo = seg * vps * 4
-            first[lo:min(lo + vps * 2, V)] = True
-            rows[::7, lo + vps * 2:min(lo + vps * 4, V)] += 20.0 / 2
-        for row in rows[::7]:      # what the first half bounds from below does not fit the tables (2048), so there is a second bound
-            assert (row >= np.sort(row[first])[-50]).sum() > 2048
+        segment = V // (16 * S)
+        for row in rows[::7]:
+            at = int(rng.integers(0, 16 * S)) * segment
+            row[at + rng.choice(segment, 2500, replace=False)] += 20.0
+            bound = np.sort(group_maxima(row, S, per_warp))[-k]
+            assert bound < 10.0 and (row >= bound).sum() > 2048
         ctx.set_cluster_size(S)
         try:
-            for k, p in ((50, 1.0), (50, 0.9)):
-                check(oracle, rows, 1.0, k, p, gpu_threshold(ctx, rows, 1.0, k, p), "S=%d k=%d p=%g" % (S, k, p))
+            for p in (1.0, 0.9):
+                check(oracle, rows, 1.0, k, p, gpu_threshold(ctx, rows, 1.0, k, p), "S=%d p=%g" % (S, p))
         finally:
             ctx.set_cluster_size(0)
