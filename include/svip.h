@@ -187,12 +187,12 @@ int svip_draft_step_at(svip_ctx* ctx, const void* logits, svip_dtype dtype, int 
  * order of summation) and may differ from an fp64 evaluation where the running
  * mass comes within about 1e-6 of top_p.  T > 0.  NaN logits count as -inf.
  * Cost: with a small top_k (at most a quarter of the threads that share a row,
- * i.e. 128 .. 1024), with or without top_p, and with top_p alone on rows that
- * are not nearly flat (up to 2048 tokens of mass above (1 - top_p) / V, of
- * which at most 1024 in the part of one of several thread blocks), every row
- * is read twice; otherwise once per radix pass:
- * 2 (bf16) or 4 (fp32) passes for top-k, as many again for the nucleus
- * (+1 for the nucleus alone).
+ * i.e. 128 .. 1024), with or without top_p, every row is read once (rows that
+ * do not fit in shared memory: and the few places in them that hold the
+ * likeliest tokens); with top_p alone on rows that are not nearly flat (up to
+ * 2048 tokens of mass above (1 - top_p) / V) twice; otherwise, and with more
+ * ties at the cut than fit, once per radix pass: 2 (bf16) or 4 (fp32) passes
+ * for top-k, as many again for the nucleus (+1 for the nucleus alone).
  *   logits  DEVICE, row r starts at element r*row_stride;  thr  DEVICE [n_rows] fp32 out
  *   stats   DEVICE [n_rows][2] fp32 out, or NULL: (m, Z) of the truncated
  *           distribution in the convention of svip_draft_step's row_stats (m the
@@ -229,8 +229,8 @@ int svip_draft_step_filtered(svip_ctx* ctx, const void* logits, svip_dtype dtype
  * thr[b] receives the threshold of row b for (top_k, top_p), and token /
  * entropy / stop / row_stats the truncated draft step at it.  With a small
  * top_k or the nucleus alone (see svip_row_threshold) the kernel finishes the
- * whole step from the few candidates it holds in shared memory, two passes over
- * the row in all; rows it cannot finish that way (flat rows, large top_k, many
+ * whole step from the few candidates it holds in shared memory, one pass over
+ * the row in all (top_p alone: two); rows it cannot finish that way (flat rows, large top_k, many
  * ties at the cut) are streamed once more at the threshold, by the same cluster.
  * Results are those of the two separate calls within the stated tolerances
  * (sums are formed in another order).

@@ -198,15 +198,16 @@ int pick_draft_cluster(const svip_ctx* ctx, long rows, int V, int dtype) {
 // Blocks per row of the threshold kernel.  Its blocks hold over 100 KB of shared memory and its rows take several
 // exchanges, so a cluster that finds no place until another one has left costs a whole second round: a size is used
 // only if all clusters fit at once, with two left as slack for the blocks of the neighbouring launches (33 clusters of 8
-// fit: 32 rows of 304 KB take 15.0 us as clusters of 8, 12.7 as clusters of 6).  Up to that the largest size of a list:
-//   top-k    powers of two, for which the groups of threads come out as just twice k (16 rows of 64 KB: 8.8 us with 2, 4
-//            or 8 blocks, 9.7 with 3, 10.6 with 6); 6 where with 4 the segments do not fit the ring (32 rows of 304 KB:
-//            12.7 us with 6, 14.0 with 4; 36 of 1 MB 16.9 and 21.1)
-//   nucleus  6, 4, 3 for long rows, 2 (16 rows of 304 KB: 10.6 us with 6, 11.5 with 8; 72 rows: 14.8 with 3, 16.2 with 2,
-//            but 9.8 and 9.5 for rows of 128 KB); 8 up to 8 rows, where it costs little and flat rows, which take the descent,
-//            gain more (8 rows of 608 KB 11.2 us with 8, 10.8 with 6, flat 42.8 and 48.1; of 512 KB 11.1 and 11.7, flat 37.1
-//            and 43.2; of 1 MB 13.8 and 12.5, flat 54.6 and 62.4; 16 rows of 608 KB 13.9 and 12.1, flat 57.4 and 55.2)
-// and 2 rather than 1 as long as it fits (144 rows of 304 KB: 18.0 against 21.4 us).  Launches that fit with no size
+// fit: 32 rows of 304 KB take 9.1 us as clusters of 8, 7.6 as clusters of 6).  Up to that the largest size of a list:
+//   top-k    powers of two (16 rows of 64 KB: 6.5 us with 2, 6.7 with 3 or 4, 7.0 with 6 or 8; 16 of 390 KB 7.3 with 8, 7.6 with 4,
+//            8.8 with 6); 6 where with 4 the segments do not fit the ring, so that stretches are fetched again (32 rows of
+//            304 KB: 7.6 us with 6, 8.8 with 4; 36 of 1 MB 12.0 and 13.7).  For 32 to 64 rows of 64 KB 2 would be faster than 4, which
+//            the list takes (6.4 and 7.2 us), for longer rows 4 (64 of 1 MB 16.1 and 17.4)
+//   nucleus  6, 4, 3 for long rows, 2 (16 rows of 304 KB: 8.6 us with 6, 9.4 with 4, 12.3 with 2; 64 of 1 MB 22.9 with 4, 25.1 with 2; 72 of
+//            128 KB 9.2 with 2 and 9.9 with 3, but 72 of 304 KB also 13.9 with 2 and 14.8 with 3); 8 up to 8 rows, for likely and flat
+//            rows alike (8 rows of 608 KB 8.6 us with 8, 8.8 with 6, flat 41.5 and 47.7; of 512 KB 7.6 and 8.5, flat 36.1 and
+//            43.7; of 1 MB 10.1 and 10.6, flat 53.6 and 63.6; but 16 rows of 608 KB 10.7 and 10.1, flat 55 either way)
+// and 2 rather than 1 as long as it fits (nucleus, 144 rows of 304 KB: 19.3 against 20.3 us).  Launches that fit with no size
 // are cut as those of the other kernels, but the nucleus alone, whose second pass over the row is as long as the first, takes 3
 // where that is at most two full rounds of blocks (rows of 384 KB up to 6/5 rows per SM, of 768 KB up to 4/3), and again from two
 // rows per SM on where the rows are so long (896 KB) that fewer blocks per row would bring more rows than L2 holds between the two

@@ -7,9 +7,9 @@
 // published definitions (top-k, nucleus sampling) read with a threshold so that the result does not
 // depend on the order of equal logits.
 //
-// One cluster per row.  Top-k with a small k and the nucleus alone take two passes and a handful of candidates (see
-// the candidate path below).  Otherwise, and where the candidates do not fit, the value is found by a radix descent over an order-preserving integer
-// image of the logits, 8 bits per pass: every pass streams the row once (cp.async ring, as the other
+// One cluster per row.  Top-k with a small k takes one pass over the row and the nucleus alone two, and a handful of candidates
+// (see the candidate path below).  Otherwise, and where the candidates do not fit, the value is found by a radix descent over
+// an order-preserving integer image of the logits, 8 bits per pass: every pass streams the row once (cp.async ring, as the other
 // kernels), histograms the digit of the elements that match the digits already fixed (counts, and
 // for the nucleus the masses 2^(l*c - M) in 2^-40 fixed point, so that every sum is an integer and
 // the result is the same whatever the order of the additions), the blocks add their histograms up
@@ -384,7 +384,7 @@ __device__ __forceinline__ unsigned long long mass_of_key(uint32_t key, float c,
 // the threshold from one pass over the row, the elements >= t0 from what the pass has left in the ring or from a second look,
 // everything else from these candidates.
 //   top-k    the maxima of disjoint groups of threads are distinct elements of the row, so the k-th largest of them
-//            is a lower bound of tau_k.  With G groups about -G ln(1 - k/G) elements lie above it (G >= 1.5 k: 1.65 k),
+//            is a lower bound of tau_k.  With G groups about -G ln(1 - k/G) elements lie above it (G = 1.5 k: 1.65 k),
 //            so the groups are made as large as that allows, which keeps the exchange and the search in it small.  The row
 //            is read once: of rows that do not fit the ring the maxima of stretches of vectors are kept, and only the
 //            stretches that reach the bound are fetched again.
@@ -396,15 +396,16 @@ __device__ __forceinline__ unsigned long long mass_of_key(uint32_t key, float c,
 //            1e-6 of top_p).
 // A segment that fits the ring (small launches) is still in shared memory for the second look.  The blocks push
 // their candidates into block 0 of the cluster, which puts up to kSorted of them in order and finds tau_k, the nucleus cut and
-// the sample by scans of one warp over the masses; in more these are found by radix descents in shared memory.  It tells the other blocks whether they are needed again.  All
-// masses are 2^-40 fixed point, so nothing depends on the order in which they are added or candidates arrive.
+// the sample by scans of one warp over the masses; in more these are found by radix descents in shared memory.  It tells the other
+// blocks whether they are needed again.  All masses are 2^-40 fixed point, so nothing depends on the order in which they are added or candidates arrive.
 // Bound by the chain of exchanges for launches of up to about 100 rows, by the pass (nucleus: the two passes) over the rows above
 // that.
 // Rows of 152064 bf16, top-k 50 + top-p 0.9, against cluster barriers with remote reads and a counting finish in every
-// block: draft step of 16 rows 18.3 -> 10.1 us, 64 rows 21.5 -> 14.3, 256 rows 41.0 -> 25.1; threshold of 2304 rows
-// 243 -> 174 us.  Top-p alone against the radix descent: 1040 rows 521 -> 91 us.  A top-k that reads its rows once, with one
-// warp's search for the bound, against two passes (of launches above 48 MB one and a half) and counting: draft step of 32 such rows
-// 12.6 -> 10.0 us, threshold of 288 rows 24.4 -> 20.7, a round of 128 sequences of 256000 fp32, 3 draft steps, 319 -> 268.
+// block, and now: draft step of 16 rows 18.3 -> 8.1 us, 64 rows 21.5 -> 11.1, 256 rows 41.0 -> 18.9; threshold of 2304 rows
+// 243 -> 124 us.  Top-p alone against the radix descent: 1040 rows 521 -> 97 us.  A top-k that reads its rows once, with one
+// warp's search for the bound and one warp's sort, against two passes (of launches above 48 MB one and a half) and counting: draft
+// step of 32 such rows 12.6 -> 8.4 us, threshold of 288 rows 24.4 -> 19.3, a round of 128 sequences of 256000
+// fp32, top-k 100, 3 draft steps, 319 -> 265.
 
 // Block-wide wait for an mbarrier of the exchange: one warp polls, the others sleep at the block barrier.
 __device__ __forceinline__ void bar_wait(unsigned long long& bar, uint32_t parity, unsigned* status, int tid) {
@@ -650,7 +651,7 @@ __device__ __forceinline__ void sample_by_index(const PoolScratch& ps, int n, ui
 // `tell` passes on to the other blocks as soon as it is certain.  A chain of dependent steps.  Up to kSorted candidates: warp 0
 // sorts the keys in registers and finds the threshold while the others put the candidates in index order by counting (80
 // candidates: 3300 cycles for both orders by counting in all warps and 5200 for the rest in one warp that read its places anew in
-// every step; 3200 in all now.  Draft step of 32 rows of 304 KB, top-k 50 + top-p 0.9, 10.0 -> 8.0 us, 8 rows of 64 KB fp32 8.6 -> 7.2).
+// every step; 3200 in all now.  Draft step of 32 rows of 304 KB, top-k 50 + top-p 0.9, 10.0 -> 8.3 us, 8 rows of 64 KB fp32 8.6 -> 7.2).
 template <int DT, bool kDraft, bool kTopK, class Tell>
 __device__ __forceinline__ uint32_t finish_pool(SelectShared& sh, PoolScratch& ps, int n, const ThresholdArgs& a, bool use_p,
                                                 unsigned long long row_mass, int row, int tid,
@@ -1054,8 +1055,10 @@ __device__ __forceinline__ void collect_mass(const RowGeom& g, const LaneSpan& s
 }
 
 // log2 of the groups of threads per warp whose maxima bound a top-k of a cluster of S blocks, if there are that many threads: in
-// the cluster at least 3/2 k groups, which leave about 1.65 k candidates; 4 k where that keeps the candidates within 128, of
-// which a warp sorts four per lane and not eight (draft step of 32 rows of 304 KB, top-k 100: 11.6 -> 9.3 us).
+// the cluster at least 3/2 k groups, which leave 1.65 to 2.1 k candidates (the search for the bound ends as soon as at most k/8
+// more than k groups reach it); 4 k, which leave 1.15 to 1.35 k, where that mostly keeps the candidates within 128, of which a warp
+// sorts four per lane and not eight (draft step of 32 rows of 304 KB, top-k 100: 11.6 -> 9.3 us).  Clusters of 3 and 6 come out at 768
+// groups there from a k of 97 on, which are more than one warp searches: a descent gives the bound.
 inline int choose_groups(int S, int k) {
     const long want = k > 64 && k <= 112 ? 4L * k : (3L * k + 1) / 2;
     int g = 0;
@@ -1190,7 +1193,7 @@ __device__ __forceinline__ uint32_t candidate_path(const RowGeom& g, const LaneS
     // kPoolCap / S candidates are pushed to block 0, which has that much room for each, and fetches the others of a block in
     // whose part of the row the likely tokens are gathered.
     Candidate* const home = kTopK ? sh.cand : sh.cand_alone;
-    const CollectInto to = S == 1 ? CollectInto{sh.landing, kPoolCap} : CollectInto{home, kTopK ? kCandPerBlock : kPoolCap};
+    const CollectInto to = S == 1 ? CollectInto{sh.landing, kPoolCap} : CollectInto{home, static_cast<uint32_t>(kTopK ? kCandPerBlock : kPoolCap)};
     const uint32_t region = kPoolCap / S;
     const bool resident = g.vps <= 32 * kStages;
     const Stretches stretches(g);
@@ -1362,7 +1365,7 @@ __global__ void __launch_bounds__(kThreads, 2) row_threshold_kernel(ThresholdArg
     RowGeom g = make_geom<DT>(rp, a.V, S * kWarps);
     const uint32_t slot0 = static_cast<uint32_t>(__cvta_generic_to_shared(ring)) + tid * 16;
     const bool use_p = a.top_p < 1.0f;
-    // a small k against the number of threads of the cluster, or the nucleus alone: two passes over the row
+    // a small k against the number of threads of the cluster, or the nucleus alone
     const bool by_candidates = kTopK ? a.top_k <= (S * kThreads) / 4 : use_p;
     const LaneSpan span = lane_span<DT>(g, rank * kWarps + warp, lane);
     if (by_candidates) candidate_open(sh, S, rank, a.groups, kTopK, tid);
