@@ -261,8 +261,14 @@ cudaError_t debug_ranges(const svip_ctx* ctx, cudaStream_t st, const void* p0, s
         r[i].hi = p[i] ? ((a + n[i] + 15ull) & ~15ull) : 0;
         if (p[i] && n[i] == ~static_cast<size_t>(0)) { r[i].lo = 0; r[i].hi = ~0ull; }   // extent not known
     }
-    if (ctx->capturing) { r[0].lo = 0; r[0].hi = ~0ull; }   // no copies from host memory into a graph
-    if (ctx->capturing) return cudaSuccess;
+    if (ctx->capturing) return cudaSuccess;      // no copies from host memory into a graph; see debug_no_ranges
+    return cudaMemcpyToSymbolAsync(g_debug_range, r, sizeof r, 0, cudaMemcpyHostToDevice, st);
+}
+// Ahead of the replay of a graph, whose buffers are not known any more: its loads are not those of the last call made singly.
+cudaError_t debug_no_ranges(cudaStream_t st) {
+    DebugRange r[2];
+    r[0].lo = r[1].lo = r[1].hi = 0;
+    r[0].hi = ~0ull;
     return cudaMemcpyToSymbolAsync(g_debug_range, r, sizeof r, 0, cudaMemcpyHostToDevice, st);
 }
 #define SVIP_DEBUG_RANGES(...) do { if (debug_ranges(__VA_ARGS__) != cudaSuccess) return SVIP_ERR_CUDA; } while (0)
@@ -1204,6 +1210,9 @@ int svip_graph_end(svip_ctx* ctx, void* stream, svip_graph** graph) {
 
 int svip_graph_launch(svip_graph* graph, void* stream) {
     if (!graph) return SVIP_ERR_INVALID_ARG;
+#ifdef SVIP_DEBUG_BOUNDS
+    if (debug_no_ranges(static_cast<cudaStream_t>(stream)) != cudaSuccess) return SVIP_ERR_CUDA;
+#endif
     return cudaGraphLaunch(graph->exec, static_cast<cudaStream_t>(stream)) == cudaSuccess ? SVIP_OK : SVIP_ERR_CUDA;
 }
 

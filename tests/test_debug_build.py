@@ -45,6 +45,25 @@ for S in (0, 1, 3):
     tl.check_draft_against_oracle(O, x, 1.0, 0.3, w.draft_uniforms[:5], got, "debug build, unaligned")
 assert ctx.read_status() == 0, "a load outside the buffers was reported"
 ctx.set_cluster_size(0)
+# a graph replayed after a call on other buffers: that call's extents are not the graph's
+x = torch.randn(2, 5000, device="cuda")
+u, z = torch.full((2,), 0.4, device="cuda"), lambda *s, d=torch.float32: torch.zeros(*s, dtype=d, device="cuda")
+single = [z(2, d=torch.int32), z(2), z(2, d=torch.uint8), z(2, 2)]
+ctx.draft_step(x, 0, 2, 5000, 5000, 1.0, 0.3, u, *single)
+replayed = [torch.zeros_like(t) for t in single]
+st = torch.cuda.Stream()
+torch.cuda.synchronize()
+ctx.graph_begin(st)
+ctx.draft_step(x, 0, 2, 5000, 5000, 1.0, 0.3, u, *replayed, st)
+graph = ctx.graph_end(st)
+other = torch.zeros(1, 64, device="cuda")
+torch.cuda.synchronize()
+ctx.draft_step(other, 0, 1, 64, 64, 1.0, 0.3, u, z(1, d=torch.int32), z(1), z(1, d=torch.uint8), z(1, 2), st)
+graph.launch(st)
+st.synchronize()
+graph.destroy()
+assert all(torch.equal(a, b) for a, b in zip(single, replayed)), (single, replayed)
+assert ctx.read_status() == 0, "loads of a replayed graph were refused"
 print("debug build ok")
 ''' % (ROOT, os.path.join(ROOT, "tests"))
 
