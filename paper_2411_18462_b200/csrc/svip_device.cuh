@@ -631,10 +631,10 @@ __device__ __forceinline__ LaneSpan lane_span(const RowGeom& g, int seg, int lan
     return s;
 }
 
-// Vectors that every lane of the warp has: n or n - 1 of each.  The streams of the threshold kernel bound their loops over whole
-// rings by it: bounded by n, the lanes that have one vector more went through a last ring while the others went through as many
-// steps of the remainder, one after the other (nucleus threshold of 64 rows of 1 MB, 31 or 32 vectors a lane: 24.2 us, now 22.8).
-// In reduce_segment() the same costs more than it gives (see there).
+// Vectors that every lane of the warp has: n or n - 1 of each.  Loops over whole rings are bounded by it: bounded by n, the lanes that
+// have one vector more went through a last ring while the others went through as many steps of the remainder, one after the other
+// (nucleus threshold of 64 rows of 1 MB, 31 or 32 vectors a lane: 24.2 us, now 22.8; draft step of 300 rows of 254 KB, 31 or 32: 27.4
+// and 24.7, of 32 rows of 304 KB, 4 or 5: 5.60 and 5.57).
 __device__ __forceinline__ int fewest_vectors(const LaneSpan& s) { return __shfl_sync(0xffffffffu, s.n, 31); }
 
 struct NeverStop { __device__ __forceinline__ bool operator()() const { return false; } };
@@ -693,6 +693,7 @@ __device__ __forceinline__ Partial reduce_segment(const RowGeom& g, const LaneSp
     // vectors that stick out of the row are folded apart, by lane 0, with their outside masked
     const bool fold_head = span.head, fold_tail = span.tail;
     const int vi0 = span.vi0, n = span.n;
+    const int full = fewest_vectors(span);
     const uint4* src = span.src;
 #pragma unroll
     for (int s = 0; s < kStages; ++s) {
@@ -735,7 +736,7 @@ __device__ __forceinline__ Partial reduce_segment(const RowGeom& g, const LaneSp
         }
         int it = 0;
         // steady state: every prefetch is in range, slot numbers are compile-time constants
-        for (; it + 2 * kStages <= n; it += kStages) {
+        for (; it + 2 * kStages <= full; it += kStages) {
             const uint4* p = src + 32 * it;
 #pragma unroll
             for (int s = 0; s < kStages; ++s) {
@@ -751,7 +752,7 @@ __device__ __forceinline__ Partial reduce_segment(const RowGeom& g, const LaneSp
             acc_check<kMode>(t, c);
         }
         // last full ring: same static slots, prefetches only where the segment still has vectors
-        for (; it + kStages <= n; it += kStages) {
+        for (; it + kStages <= full; it += kStages) {
             const uint4* p = src + 32 * it;
 #pragma unroll
             for (int s = 0; s < kStages; ++s) {
@@ -766,15 +767,14 @@ __device__ __forceinline__ Partial reduce_segment(const RowGeom& g, const LaneSp
             }
             acc_check<kMode>(t, c);
         }
-        // fewer than kStages vectors left, all of them already in flight: `it` is a multiple of
+        // at most kStages vectors left, all of them already in flight: `it` is a multiple of
         // kStages, so vector it + k sits in slot k.  Unrolled, because small launches spend their whole stream here (draft
-        // step of 16 rows of 200 KB bf16: rolled 6.0 us, unrolled 5.05; greedy round of 8 rows of 200 KB fp32, 5 steps and
-        // the verification, 23.4 and 22.2), with one test a vector (ring loops bounded by what all lanes of the warp have,
-        // and a second test per vector here: 32 rows of 304 KB 5.73 instead of 5.61, 32 such steps and a verification that
-        // stops at the first rejection 225 instead of 219).
+        // step of 16 rows of 200 KB bf16: rolled 6.0 us, unrolled 4.95; greedy round of 8 rows of 200 KB fp32, 5 steps and
+        // the verification, 23.3 and 21.5), with one test a vector (with a test for all lanes and one for each: 32 rows of
+        // 304 KB 5.74 instead of 5.57, 32 such steps and a verification that stops at the first rejection 225 instead of 218).
         cp_async_wait<0>();
 #pragma unroll
-        for (int s = 0; s < kStages - 1; ++s) {
+        for (int s = 0; s < kStages; ++s) {
             if (it + s >= n) break;
             const uint4 raw = lds128(slot0 + s * kSlotStride);
             float x[EPV];
