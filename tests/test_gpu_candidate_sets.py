@@ -1,5 +1,5 @@
-"""Large candidate sets of the threshold kernel: more group maxima and more candidates than are put in order by counting
-(256), up to what the tables hold (2048), with and without a nucleus inside the top-k; and that such a call costs a small
+"""Large candidate sets of the threshold kernel: more group maxima than one warp searches (512) and more candidates than
+it sorts (256), up to what the tables hold (2048), with and without a nucleus inside the top-k; and that such a call costs a small
 multiple of a small top-k and not its square.  Oracle and tolerances are those of test_gpu_truncation."""
 import numpy as np
 import pytest
